@@ -292,6 +292,8 @@ struct LegTerms {
   float nde;      // gam sig / (r - a sig)^2
   float phi;      // phi2(r)
   float dphi;     // dphi2 / dr
+  float t, ae2;   // 1 / (r - a sig), A eps exp(sig / (r - a sig)) (the adjoint's second derivative)
+  float invu;     // 1 / |d| of the unstretched d (kFine): u = d invu
 };
 
 // 1/x from the hardware approximation (rcp.approx.ftz: within one ulp); the
@@ -316,12 +318,38 @@ __device__ __forceinline__ float ex2_approx(float x) {
   return y;
 }
 
-template <class C>
-__device__ __forceinline__ bool leg_terms(float r2, const C& c, LegTerms& o) {
+// 2^(a + al), a <= 0 and al its low part, by the Taylor series of 2^f at the
+// nearest integer (|f| <= 1/2, seven terms: truncation 5e-9), without the
+// hardware approximation's bias, which is the same sign for every leg and so
+// survives a sum over all of them.  Below 2^-126: 0 (ex2_approx flushes too).
+__device__ __forceinline__ float exp2_taylor(float a, float al) {
+  const float n = rintf(a);
+  const float f = (a - n) + al;
+  float p = 1.5252734e-5f;  // (ln 2)^k / k!, k = 7 ... 1
+  p = fmaf(p, f, 1.5403530e-4f);
+  p = fmaf(p, f, 1.3333558e-3f);
+  p = fmaf(p, f, 9.6181291e-3f);
+  p = fmaf(p, f, 5.5504109e-2f);
+  p = fmaf(p, f, 2.4022651e-1f);
+  p = fmaf(p, f, 6.9314718e-1f);
+  p = fmaf(p, f, 1.0f);
+  return n < -125.0f ? 0.0f : p * __int_as_float(((int)n + 127) << 23);
+}
+
+// kFine (the adjoint, whose parameter derivatives are sums of one sign over
+// all legs): the exponentials by exp2_taylor instead of the hardware
+// approximation, and the leg's length stretched by the relative amount
+// `stretch` (below an FP32 ulp, so it goes into the low part dr).
+template <bool kFine = false, class C>
+__device__ __forceinline__ bool leg_terms(float r2, const C& c, LegTerms& o, float stretch = 0.f) {
   constexpr float kLn2 = 0.693147180559945f;
   const float v = rsqrt_approx(r2);
   const float r = r2 * v;
-  const float dr = 0.5f * fmaf(-r, r, r2) * v;
+  float dr = 0.5f * fmaf(-r, r, r2) * v;
+  if constexpr (kFine) {
+    o.invu = fmaf(v, fmaf(-r, v, 1.0f) - dr * v, v);
+    dr = fmaf(r, stretch, dr);
+  }
   if (!(r + dr < c.rc)) return false;
   const float ev = fmaf(-r, v, 1.0f) - dr * v;
   const float xh = r - c.rc;
@@ -330,12 +358,21 @@ __device__ __forceinline__ bool leg_terms(float r2, const C& c, LegTerms& o) {
   const float tc = fmaf(-xh, t, 1.0f) - xl * t;
   const float a2 = c.sig_l2e * t;
   const float a2l = fmaf(c.sig_l2e, t, -a2) + fmaf(a2, tc, c.sig_l2e_lo * t);
-  float e2 = ex2_approx(a2);
-  e2 = fmaf(e2, kLn2 * a2l, e2);
+  float e2;
+  if constexpr (kFine) {
+    e2 = exp2_taylor(a2, a2l);
+  } else {
+    e2 = ex2_approx(a2);
+    e2 = fmaf(e2, kLn2 * a2l, e2);
+  }
   const float a3 = c.gsig_l2e * t;
   const float a3l = fmaf(c.gsig_l2e, t, -a3) + fmaf(a3, tc, c.gsig_l2e_lo * t);
-  const float e3 = ex2_approx(a3);
-  o.e3 = fmaf(e3, kLn2 * a3l, e3);
+  if constexpr (kFine) {
+    o.e3 = exp2_taylor(a3, a3l);
+  } else {
+    const float e3 = ex2_approx(a3);
+    o.e3 = fmaf(e3, kLn2 * a3l, e3);
+  }
   const float invr = fmaf(v, ev, v);
   const float t2 = t * t;
   const float t2l = fmaf(t, t, -t2) + 2.0f * t2 * tc;  // t^2 (1 + 2 tc) = t2 + t2l
@@ -343,6 +380,8 @@ __device__ __forceinline__ bool leg_terms(float r2, const C& c, LegTerms& o) {
   o.invr = invr;
   o.nde = c.gsig * fmaf(t2, 2.0f * tc, t2);
   const float ae2 = c.Aeps * e2;
+  o.t = fmaf(t, tc, t);
+  o.ae2 = ae2;
   if (c.p == 4 && c.q == 0) {
     // u = sig / r, y = B u^4, each as hi + lo
     const float uh = c.sig * v;
@@ -1086,7 +1125,6 @@ constexpr int kG = 4;                    // lanes per centre in the leg phase
 constexpr int kFThreads = 128;
 constexpr int kFAtoms = kFThreads / kG;  // centres per block
 constexpr int kWAtoms = 32 / kG;         // centres per warp
-constexpr int kLPad = kLMax + 1;         // row pitch (float4) of the adjoint's leg tables
 constexpr int kPre = 6;                  // neighbour slots per lane fetched ahead in the leg phase (8 spills at 64 registers)
 
 // The force kernel's shared-memory leg table: a row of kRow float4 records
@@ -1202,6 +1240,69 @@ __device__ __noinline__ void force_overflow_item(const Dev& d, const FParams& P,
   for (int k = 0; k < 6; ++k) atomicAdd(p + 2 + k, (double)w[k]);
 }
 
+// Leg phase A of one species (k_force and the adjoint): the KG lanes of a
+// centre walk its neighbour row and compact the pairs with r^2 < rc2 into the
+// centre's leg records tab(l) = (d, j), at most kLM of them; returns how many
+// there are.  Row entries and candidate positions are fetched for kPre slots
+// per lane before any is used (two memory latencies per batch instead of a
+// dependent chain per slot); every slot's test comes first, then one
+// compaction per batch (the lane's hits go to the group's running count plus
+// the hits of the group's lower lanes in this batch, in slot order).  Rows
+// longer than KG * kPre cost one more round trip per batch, not per slot.
+// Every lane of the warp calls it.
+template <int KG, int kLM, class At>
+__device__ __forceinline__ int stage_legs(const Dev& d, float rc2, float4* tab, At at, const uint4& qi, float L0, float L1,
+                                          float L2, const int* row, int cnt) {
+  const int lane = threadIdx.x & 31;
+  const int g = threadIdx.x & (KG - 1);
+  const int iters = __reduce_max_sync(kFull, (cnt + KG - 1) / KG);
+  int nl = 0;
+  for (int t0 = 0; t0 < iters; t0 += kPre) {  // warp-uniform
+    int jr[kPre];
+    uint32_t qx[kPre], qy[kPre], qz[kPre];
+#pragma unroll
+    for (int t = 0; t < kPre; ++t) {
+      const int s = g + KG * (t0 + t);
+      jr[t] = (s < cnt) ? row[s] : -1;
+    }
+#pragma unroll
+    for (int t = 0; t < kPre; ++t) {
+      uint4 qj = make_uint4(0u, 0u, 0u, 0u);
+      if (jr[t] >= 0) qj = d.q[jr[t]];
+      qx[t] = qj.x;
+      qy[t] = qj.y;
+      qz[t] = qj.z;
+    }
+    float dx[kPre], dy[kPre], dz[kPre];
+    unsigned hits = 0u;  // bit t: slot t is a leg
+    int hc = 0;
+#pragma unroll
+    for (int t = 0; t < kPre; ++t) {
+      dx[t] = fix_diff(qi.x, qx[t], L0);
+      dy[t] = fix_diff(qi.y, qy[t], L1);
+      dz[t] = fix_diff(qi.z, qz[t], L2);
+      const bool hit = jr[t] >= 0 && fmaf(dx[t], dx[t], fmaf(dy[t], dy[t], dz[t] * dz[t])) < rc2;
+      hits |= hit ? 1u << t : 0u;
+      hc += hit ? 1 : 0;
+    }
+    int incl = hc;  // inclusive prefix of the hit counts over the group's lanes
+#pragma unroll
+    for (int o = 1; o < KG; o <<= 1) {
+      const int y = __shfl_up_sync(kFull, incl, o, KG);
+      if (g >= o) incl += y;
+    }
+    int pos = nl + incl - hc;
+#pragma unroll
+    for (int t = 0; t < kPre; ++t)
+      if ((hits >> t) & 1u) {
+        if (pos < kLM) tab[at(pos)] = make_float4(dx[t], dy[t], dz[t], __int_as_float(jr[t]));
+        ++pos;
+      }
+    nl += __shfl_sync(kFull, incl, lane | (KG - 1));  // the group's hits in this batch
+  }
+  return nl;
+}
+
 template <bool kCount>
 __device__ __noinline__ int species_item(const Dev& d, const SpPair* sp, const float2* st, int nsp, int i,
                                          float (&acc)[8]);
@@ -1258,41 +1359,11 @@ __device__ void force_block(const Dev& d, const FParams& P,
       spi = sps + ti * nsp;
     }
   }
-  // ---- leg phase A: row entries and candidate positions are fetched for
-  // kPre slots per lane before any is used (two memory latencies per batch
-  // instead of a dependent chain per slot).  Distance test only; hits are
-  // compacted (ballot + popc in the lane group) into the centre's row as one
-  // record (d, j) (several species: (d, r^2) and (species, j)).
-  const int iters = __reduce_max_sync(kFull, (cnt + KG - 1) / KG);
-  const unsigned gsh = lane & ~(KG - 1);
+  // ---- leg phase A (stage_legs).  Several species: each candidate is tested
+  // against its own pair's cutoff, slot by slot (ballot + popc in the lane
+  // group), and its record is (d, r^2) and (species, j).
   const int* row = d.nbr + (size_t)(valid ? i : 0) * d.W;
   int nl = 0;
-  // (kSp: the partner's species rides in the record's x slot until phase B)
-  auto test_slot = [&](int j, uint32_t jx, uint32_t jy, uint32_t jz, int tj, bool have) {
-    bool hit = false;
-    float dx = 0.f, dy = 0.f, dz = 0.f, r2 = 0.f;
-    if (have) {
-      dx = fix_diff(qi.x, jx, L0);
-      dy = fix_diff(qi.y, jy, L1);
-      dz = fix_diff(qi.z, jz, L2);
-      r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-      if constexpr (kSp)
-        hit = r2 < spi[tj].rc2;
-      else
-        hit = r2 < P.rc2;
-    }
-    const unsigned m = (__ballot_sync(kFull, hit) >> gsh) & ((1u << KG) - 1u);
-    const int pos = nl + __popc(m & ((1u << g) - 1u));
-    if (hit && pos < kLM) {
-      if constexpr (kSp) {  // (the pair's cutoff test needs r^2 again in phase B: kept)
-        T.ue[at(pos)] = make_float4(dx, dy, dz, r2);
-        T.aux[at(pos)] = make_float4(__int_as_float(tj), 0.f, 0.f, __int_as_float(j));
-      } else {  // one record: r^2 is recomputed from d in phase B by the same expression
-        T.ue[at(pos)] = make_float4(dx, dy, dz, __int_as_float(j));
-      }
-    }
-    nl += __popc(m);
-  };
   if constexpr (kOwn == 2) {  // the legs pass 1 staged, their vectors recomputed
     const int nlg = valid ? d.nleg[i] : 0;
     nl = nlg < 0 ? 0 : nlg;
@@ -1302,64 +1373,51 @@ __device__ void force_block(const Dev& d, const FParams& P,
       const float dx = fix_diff(qi.x, qj.x, L0), dy = fix_diff(qi.y, qj.y, L1), dz = fix_diff(qi.z, qj.z, L2);
       T.ue[at(l)] = make_float4(dx, dy, dz, __int_as_float(j));
     }
-  } else
-  // batches of kPre slots per lane, each fetched as a whole (rows, then
-  // positions) before its tests: rows longer than KG * kPre cost one more
-  // round trip per batch, not per slot
-  for (int t0 = 0; t0 < iters; t0 += kPre) {  // warp-uniform
-    int jr[kPre];
-    uint32_t qx[kPre], qy[kPre], qz[kPre];
-    int tj[kPre];
-#pragma unroll
-    for (int t = 0; t < kPre; ++t) {
-      const int s = g + KG * (t0 + t);
-      jr[t] = (s < cnt) ? row[s] : -1;
-    }
-#pragma unroll
-    for (int t = 0; t < kPre; ++t) {
-      uint4 qj = make_uint4(0u, 0u, 0u, 0u);
-      if (jr[t] >= 0) qj = d.q[jr[t]];
-      qx[t] = qj.x;
-      qy[t] = qj.y;
-      qz[t] = qj.z;
-      tj[t] = 0;
-      if constexpr (kSp)
-        if (jr[t] >= 0) tj[t] = d.typ[jr[t]];
-    }
-    if constexpr (kSp == 0) {
-      // one species: every slot's test first, then one compaction per batch
-      // (the lane's hits go to the group's running count plus the hits of the
-      // group's lower lanes in this batch, in slot order)
-      float dx[kPre], dy[kPre], dz[kPre];
-      unsigned hits = 0u;  // bit t: slot t is a leg
-      int hc = 0;
+  } else if constexpr (kSp == 0) {
+    nl = stage_legs<KG, kLM>(d, P.rc2, T.ue, at, qi, L0, L1, L2, row, cnt);
+  } else {
+    const int iters = __reduce_max_sync(kFull, (cnt + KG - 1) / KG);
+    const unsigned gsh = lane & ~(KG - 1);
+    for (int t0 = 0; t0 < iters; t0 += kPre) {  // warp-uniform
+      int jr[kPre], tj[kPre];
+      uint32_t qx[kPre], qy[kPre], qz[kPre];
 #pragma unroll
       for (int t = 0; t < kPre; ++t) {
-        dx[t] = fix_diff(qi.x, qx[t], L0);
-        dy[t] = fix_diff(qi.y, qy[t], L1);
-        dz[t] = fix_diff(qi.z, qz[t], L2);
-        const bool hit = jr[t] >= 0 && fmaf(dx[t], dx[t], fmaf(dy[t], dy[t], dz[t] * dz[t])) < P.rc2;
-        hits |= hit ? 1u << t : 0u;
-        hc += hit ? 1 : 0;
+        const int s = g + KG * (t0 + t);
+        jr[t] = (s < cnt) ? row[s] : -1;
       }
-      int incl = hc;  // inclusive prefix of the hit counts over the group's lanes
 #pragma unroll
-      for (int o = 1; o < KG; o <<= 1) {
-        const int y = __shfl_up_sync(kFull, incl, o, KG);
-        if (g >= o) incl += y;
-      }
-      int pos = nl + incl - hc;
-#pragma unroll
-      for (int t = 0; t < kPre; ++t)
-        if ((hits >> t) & 1u) {
-          if (pos < kLM) T.ue[at(pos)] = make_float4(dx[t], dy[t], dz[t], __int_as_float(jr[t]));
-          ++pos;
+      for (int t = 0; t < kPre; ++t) {
+        uint4 qj = make_uint4(0u, 0u, 0u, 0u);
+        tj[t] = 0;
+        if (jr[t] >= 0) {
+          qj = d.q[jr[t]];
+          tj[t] = d.typ[jr[t]];
         }
-      nl += __shfl_sync(kFull, incl, lane | (KG - 1));  // the group's hits in this batch
-    } else {
+        qx[t] = qj.x;
+        qy[t] = qj.y;
+        qz[t] = qj.z;
+      }
 #pragma unroll
-      for (int t = 0; t < kPre; ++t)
-        if (t0 + t < iters) test_slot(jr[t], qx[t], qy[t], qz[t], tj[t], jr[t] >= 0);
+      for (int t = 0; t < kPre; ++t) {
+        if (t0 + t >= iters) break;
+        bool hit = false;
+        float dx = 0.f, dy = 0.f, dz = 0.f, r2 = 0.f;
+        if (jr[t] >= 0) {
+          dx = fix_diff(qi.x, qx[t], L0);
+          dy = fix_diff(qi.y, qy[t], L1);
+          dz = fix_diff(qi.z, qz[t], L2);
+          r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+          hit = r2 < spi[tj[t]].rc2;
+        }
+        const unsigned m = (__ballot_sync(kFull, hit) >> gsh) & ((1u << KG) - 1u);
+        const int pos = nl + __popc(m & ((1u << g) - 1u));
+        if (hit && pos < kLM) {  // (the pair's cutoff test needs r^2 again in phase B: kept)
+          T.ue[at(pos)] = make_float4(dx, dy, dz, r2);
+          T.aux[at(pos)] = make_float4(__int_as_float(tj[t]), 0.f, 0.f, __int_as_float(jr[t]));
+        }
+        nl += __popc(m);
+      }
     }
   }
   __syncwarp();

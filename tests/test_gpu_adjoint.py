@@ -140,3 +140,36 @@ def test_autograd_force_matching_step(mwlib, orc):
     gx_ref, gt_ref = orc.force_vjp(x, box, w, po)
     assert _rel_err_rows(gx, gx_ref) <= G_TOL
     _check_theta(orc, x, box, w, gth, gt_ref, po)
+
+
+EDGES = {
+    # one leg per centre (no three-body term), three atoms (each centre two legs)
+    "pair": (lambda: (np.array([[1.0, 2.0, 3.0], [3.2, 3.5, 4.0]]), np.array([20.0, 22.0, 25.0])), {}),
+    "triplet": (lambda: (np.array([[0.2, 0.1, 0.3], [2.6, 0.4, 0.1], [24.6, 2.9, 0.2]]), np.array([25.0, 22.0, 21.0])),
+                {}),
+    # last block of 32 centres holding one atom; three different edges
+    "block_edge_257": (lambda: (I.lattice_fill(257, [0, 0, 0], [19.0, 20.0, 20.5], 1.0, 0.2, 31),
+                                np.array([19.0, 20.0, 20.5])), {}),
+    # the general pair exponents
+    "p6_q1_500": (lambda: I.jittered_box(500, 1.0, 0.2, 32), {"p": 6, "q": 1}),
+}
+
+
+@pytest.mark.parametrize("case", sorted(EDGES))
+def test_adjoint_edges_match_oracle(mwlib, orc, case):
+    torch = pytest.importorskip("torch")
+    make, kw = EDGES[case]
+    x, box = make()
+    x = I.snap_to_grid(x, box)
+    w = np.random.default_rng(14).normal(size=x.shape)
+    gx_ref, gt_ref = orc.force_vjp(x, box, w, orc.params(**kw))
+    prm = mwlib.mw_params_default()
+    for k, v in kw.items():
+        setattr(prm, k, v)
+    gx, gt = _gpu_vjp(mwlib, torch, len(x), box, x, w, prm)
+    assert _rel_err_rows(gx, gx_ref) <= G_TOL
+    if len(x) == 2:  # no three-body term: its derivative is exactly zero
+        assert gt[0][0] == 0.0 and abs(gt_ref[0]) < 1e-12
+        assert np.allclose(gt[0][1:], gt_ref[1:], rtol=G_TOL)
+    else:
+        _check_theta(orc, x, box, w, gt[0], gt_ref, orc.params(**kw))
