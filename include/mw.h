@@ -82,7 +82,9 @@ typedef enum mw_thermostat { MW_NVE = 0, MW_BERENDSEN = 1, MW_NOSE_HOOVER = 2, M
 
 /* How mw_step launches work.  GRAPH: one kernel per phase, one step captured
  * in a CUDA graph and replayed.  PERSISTENT: one cooperative launch runs many
- * steps with grid-wide barriers between phases.  AUTO: the library picks
+ * steps with grid-wide barriers between phases; mw_step runs small boxes, and
+ * batches of them, in one thread-block cluster per box instead (the library
+ * picks by size; same results to rounding).  AUTO: the library picks
  * (the autotuner's choice when one was made, else PERSISTENT).  PLAIN: the
  * plain GPU path the others are measured against: every phase kernel
  * launched from the host every step (no graph, no persistent launch) and a

@@ -7,12 +7,14 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <array>
 #include <atomic>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -21,6 +23,7 @@
 #include "mw.h"
 #include "mw_device.cuh"
 #include "mw_persistent.cuh"
+#include "mw_cluster.cuh"
 #include "mw_adjoint.cuh"
 #include "mw_structure.cuh"
 #include "mw_species.cuh"
@@ -115,6 +118,9 @@ struct mw_system {
   int pers_blocks = 0;
   int pers_blocks_limit = 0;  // 0 = as many as can be co-resident
   unsigned long long wait_ns = kBarrierTimeoutNs;  // limit of each device-side wait
+  // its cluster form: one buffer for the box order and the per-box progress
+  int* clu_order = nullptr;
+  bool clu_resume = false;  // the next launch goes on with boxes that stopped on their own steps
   std::vector<int> cell_box_host;
   std::vector<void*> allocs;
   // pinned host staging for the small device-to-host reads (the Global
@@ -1151,6 +1157,7 @@ mw_status create_common(mw_system** out, int nbox, const int* n, const double* b
 }  // namespace
 
 #include "mw_persistent_host.inc"
+#include "mw_cluster_host.inc"
 #include "mw_adjoint_host.inc"
 #include "mw_autotune.inc"
 #include "mw_structure_host.inc"
@@ -1525,8 +1532,11 @@ mw_status mw_step(mw_system* s, const mw_integrator* integ, int nsteps, mw_therm
     if (eng == MW_ENGINE_AUTO) eng = s->tuned_engine >= 0 ? s->tuned_engine : MW_ENGINE_PERSISTENT;
     if (eng == MW_ENGINE_PERSISTENT && !persistent_available(s)) eng = MW_ENGINE_GRAPH;
     s->engine_used = eng;
-    st = eng == MW_ENGINE_PERSISTENT ? run_persistent_engine(s, nsteps, last, &fetched)
-                                     : run_graph_engine(s, nsteps, last, &fetched, eng == MW_ENGINE_PLAIN);
+    CluConfig clu;
+    st = eng == MW_ENGINE_PERSISTENT
+             ? (cluster_config(s, &clu) ? run_cluster_engine(s, clu, nsteps, last, &fetched)
+                                        : run_persistent_engine(s, nsteps, last, &fetched))
+             : run_graph_engine(s, nsteps, last, &fetched, eng == MW_ENGINE_PLAIN);
     s->g_known_valid = false;
     if (st != MW_OK) {
       s->forces_valid = false;  // the state of an interrupted step is not a state to report forces of

@@ -48,18 +48,18 @@ struct Box {        // read-only in kernels, except the geometry under isobaric 
   double dtL[3];    // dt / L: drift of the box fraction per unit velocity
   float dtL64[3];   // dt / L * 2^64: drift in 2^-64 box-fraction units per unit velocity (FP32)
   float lost;       // half the shortest edge (A)
-  double qs[3];     // 2^32 / L
+  double qs[3];     // unused (2^32 / L at creation; checkpoints hold this structure)
   float Lq[3];      // L / 2^32
   int off, n;       // atom range
   int nc[3];        // cells per dimension
   int cell_off;     // first global cell
   double T0, Ndf, Q, volume;
-  double invQ;      // 1 / Q
+  double invQ;      // unused (1 / Q)
   double ndfkT0;    // N_df k_B T0
   double q4;        // dt / (4 Q): quarter-step factor of xi
   float q4f;        // q4 in FP32
   double inv_ndf_kb;  // 1 / (N_df k_B): T = 2 KE inv_ndf_kb
-  double p_fac;     // atm per kcal/mol of 2 KE + tr W: 1/(3 V) in atm
+  double p_fac;     // unused (1/(3 V) in atm at creation)
   int vexp_lost;    // a velocity component whose FP32 exponent field is >= this is a runaway (see validate_integ)
   // isobaric runs only: the box scales at the drift of every step
   float hs2;        // squared displacement (measured with this step's Lq) that triggers a rebuild
@@ -646,17 +646,42 @@ __device__ void write_record(const Dev& d, const Integ& I, int b, int pp, unsign
   for (int k = 0; k < 3; ++k) r[TR_L0 + k] = bx.L[k];
 }
 
+// How the end-of-step tails read what an earlier phase wrote: with L2 loads
+// from global memory (another block may have written it in the same launch),
+// or plainly from the block's own shared copy (the cluster engine).
+struct LdGlobal {
+  template <class T>
+  __device__ static T get(const T& v) { return __ldcg(&v); }
+};
+struct LdShared {
+  template <class T>
+  __device__ static T get(const T& v) { return v; }
+};
+
+// a / b (FP64) from an FP32 reciprocal and two Newton steps: relative error
+// below 1e-13 in five FP64 operations.  The library division takes several
+// times that, and GB300 issues an FP64 instruction every ~25 cycles even for
+// one lane: with five divisions the isobaric tail took 5.5 us per step.  Its
+// callers round the quotient to FP32.  Divisors outside FP32's range divide.
+__device__ __forceinline__ double div_newton(double a, double b) {
+  const float bf = (float)b;
+  if (!(fabsf(bf) > 1e-30f && fabsf(bf) < 1e30f)) return a / b;
+  double r = (double)__frcp_rn(bf);
+  r = fma(r, fma(-b, r, 1.0), r);
+  r = fma(r, fma(-b, r, 1.0), r);
+  return a * r;
+}
+
 // Isotropic barostat (Sec. II.B, read as the Martyna-Tobias-Klein form):
 // half step on its momentum, pe += dt/2 [(1 + 3/N_df) 2 KE + tr(W) - 3 P V],
 // and the friction on the velocities, v *= exp(-dt/2 (1 + 3/N_df) pe/W),
-// returned as s - 1 (FP32).  pe and the volume stay FP64.  The geometry is
-// read with L2 loads (__ldcg): in the persistent engine another block wrote
-// it earlier in the same launch.
+// returned as s - 1 (FP32).  pe and the volume stay FP64.
+template <class Ld = LdGlobal>
 __device__ __forceinline__ void baro_half(const Integ& I, const Box& bx, double ke, double trw, double& pe) {
-  pe += 0.5 * I.dt * (bx.a3 * 2.0 * ke + trw - 3.0 * I.p_ext * __ldcg(&bx.volume));
+  pe += 0.5 * I.dt * (bx.a3 * 2.0 * ke + trw - 3.0 * I.p_ext * Ld::get(bx.volume));
 }
 __device__ __forceinline__ float baro_friction(const Integ& I, const Box& bx, double pe) {
-  return expm1f((float)(-0.5 * I.dt * bx.a3 * pe / bx.W));
+  return expm1f((float)div_newton(-0.5 * I.dt * bx.a3 * pe, bx.W));
 }
 
 // The box of the coming step: every edge scaled by e^u, u = dt pe/W, during
@@ -669,103 +694,108 @@ __device__ __forceinline__ float baro_friction(const Integ& I, const Box& bx, do
 // since the build, so the list holds while 2 d <= r_list - r_c -
 // r_list max(0, 1 - c); the displacement is measured with the current
 // edges, e^-u of the new ones.  A margin below skin/2 rebuilds at once.
-__device__ void npt_geometry(const Dev& d, const Integ& I, int b, double pe) {
-  Box& bx = const_cast<Box*>(d.box)[b];
-  BoxState* st = d.bst + b;
-  const float u = (float)(I.dt * pe / bx.W);
+// Returns bit 0: the margin asks for a rebuild, bit 1: the box left its grid.
+template <class Ld>
+__device__ int npt_geometry_of(const Integ& I, Box& bx, BoxState& st, double pe) {
+  const float u = (float)div_newton(I.dt * pe, bx.W);
   const float eu = expm1f(u);
   const float fdr = fabsf(u) > 1e-3f ? -expm1f(-u) / u : fmaf(u, fmaf(u, 1.0f / 6.0f, -0.5f), 1.0f);
   const float dt64 = (float)(I.dt * 18446744073709551616.0);  // dt 2^64
-  bool grid = false;
+  int out = 0;
   for (int k = 0; k < 3; ++k) {
-    const double L = __ldcg(&bx.L[k]);
+    const double L = Ld::get(bx.L[k]);
     const double Ln = fma(L, (double)eu, L);
     bx.dtL64[k] = dt64 / (float)L * fdr;
     bx.Ln[k] = Ln;
     const int nc = bx.nc[k];
-    if (Ln < 2.0 * I.rlist || (nc >= 4 && Ln < nc * (double)I.rlist) || Ln >= (nc + 1) * kCellGrow * I.rlist)
-      grid = true;
+    if (Ln < 2.0 * I.rlist || (nc >= 4 && Ln < nc * (double)I.rlist) || Ln >= (nc + 1) * kCellGrow * I.rlist) out = 2;
   }
-  if (grid) set_status(d.g, ST_GRID);
-  const float c = (float)(bx.Ln[0] / __ldcg(&st->Lb));
+  const float c = (float)div_newton(bx.Ln[0], Ld::get(st.Lb));
   const float m = I.skin - I.rlist * fmaxf(0.0f, 1.0f - c);
   if (m < 0.5f * I.skin) {
-    st->rebuild = 1;
-    d.g->any_rebuild = 1;
+    st.rebuild = 1;
+    out |= 1;
   }
   const float h = 0.5f * fmaxf(m, 0.0f) / (1.0f + eu);
   bx.hs2 = h * h;
+  return out;
+}
+__device__ void npt_geometry(const Dev& d, const Integ& I, int b, double pe) {
+  const int r = npt_geometry_of<LdGlobal>(I, const_cast<Box*>(d.box)[b], d.bst[b], pe);
+  if (r & 2) set_status(d.g, ST_GRID);
+  if (r & 1) d.g->any_rebuild = 1;
 }
 
 // The edges of the coming step made current (the last block of kick1, once
 // every block has drifted with the old ones).
-__device__ void npt_commit_box(const Dev& d, int b) {
-  Box& bx = const_cast<Box*>(d.box)[b];
+template <class Ld>
+__device__ void npt_commit(Box& bx) {
   double vol = 1.0;
   for (int k = 0; k < 3; ++k) {
-    const double Ln = __ldcg(&bx.Ln[k]);
+    const double Ln = Ld::get(bx.Ln[k]);
     bx.L[k] = Ln;
     bx.Lq[k] = (float)(Ln * 2.3283064365386963e-10);  // 2^-32
-    bx.qs[k] = 4294967296.0 / Ln;
     vol *= Ln;
   }
   bx.volume = vol;
-  bx.p_fac = kATM / (3.0 * vol);
+}
+__device__ void npt_commit_box(const Dev& d, int b) { npt_commit<LdGlobal>(const_cast<Box*>(d.box)[b]); }
+
+// Thermostat at the end of a step, for one box (after the step's kinetic-
+// energy sum ke0 is complete): the end half of this step, then the start half
+// of the next one; stores the state after each half and the combined scale
+// S - 1 the next kick1 applies.  Isobaric (kNpt instantiations only, so that
+// the FP64 barostat arithmetic does not raise the register count of the
+// others; trw the trace of the step's virial): friction, barostat half,
+// thermostat half end this step; thermostat half, barostat half, friction
+// start the next; then the new box.  Returns npt_geometry_of's bits.
+template <bool kNpt, class Ld>
+__device__ int end_of_step(const Integ& I, Box& bx, BoxState& st, double ke0, double trw) {
+  if constexpr (kNpt) {
+    double pe = Ld::get(st.pe_b);
+    const float f1 = baro_friction(I, bx, pe);
+    double ke = fma(ke0, (double)(f1 * (2.0f + f1)), ke0);
+    baro_half<Ld>(I, bx, ke, trw, pe);
+    ThermoState t = thermo_in(bx, Ld::get(st.th), ke);
+    const float se = end_half<true>(I, bx, t);
+    ke = fma(ke, (double)(se * (2.0f + se)), ke);
+    st.th_e = make_float4(t.xh, t.xl, t.eh, t.el);
+    st.ke_last = ke;
+    st.pe_e = pe;
+    const float e1 = fmaf(f1, se, f1 + se);
+    st.s_endc = 1.0 + (double)e1;
+    const float ss = start_half<true>(I, bx, t);
+    ke = fma(ke, (double)(ss * (2.0f + ss)), ke);
+    st.th = make_float4(t.xh, t.xl, t.eh, t.el);
+    baro_half<Ld>(I, bx, ke, trw, pe);
+    const float f2 = baro_friction(I, bx, pe);
+    const float e2 = fmaf(ss, f2, ss + f2);
+    st.sig = fmaf(e1, e2, e1 + e2);
+    st.pe_b = pe;
+    return npt_geometry_of<Ld>(I, bx, st, pe);
+  } else {
+    ThermoState t = thermo_in(bx, Ld::get(st.th), ke0);
+    const float se = end_half(I, bx, t);
+    st.th_e = make_float4(t.xh, t.xl, t.eh, t.el);
+    st.ke_last = fma(ke0, (double)(se * (2.0f + se)), ke0);
+    st.s_endc = 1.0 + (double)se;
+    const float ss = start_half(I, bx, t);
+    st.th = make_float4(t.xh, t.xl, t.eh, t.el);
+    st.sig = fmaf(se, ss, se + ss);
+    return 0;
+  }
 }
 
-// Isobaric end-of-step tail (kNpt instantiations only, so that the FP64
-// barostat arithmetic does not raise the register count of the others).
-__device__ void end_of_step_box_npt(const Dev& d, const Integ& I, int b, int par) {
-  BoxState* st = d.bst + b;
-  const Box& bx = d.box[b];
-  const double ke0 = __ldcg(&st->ke_acc[par]);
-  // end of this step: friction, barostat half, thermostat half; start of
-  // the next: thermostat half, barostat half, friction; then the new box
-  const double trw = __ldcg(&st->ew[par][2]) + __ldcg(&st->ew[par][3]) + __ldcg(&st->ew[par][4]);
-  double pe = __ldcg(&st->pe_b);
-  const float f1 = baro_friction(I, bx, pe);
-  double ke = fma(ke0, (double)(f1 * (2.0f + f1)), ke0);
-  baro_half(I, bx, ke, trw, pe);
-  ThermoState t = thermo_in(bx, __ldcg(&st->th), ke);
-  const float se = end_half<true>(I, bx, t);
-  ke = fma(ke, (double)(se * (2.0f + se)), ke);
-  st->th_e = make_float4(t.xh, t.xl, t.eh, t.el);
-  st->ke_last = ke;
-  st->pe_e = pe;
-  const float e1 = fmaf(f1, se, f1 + se);
-  st->s_endc = 1.0 + (double)e1;
-  const float ss = start_half<true>(I, bx, t);
-  ke = fma(ke, (double)(ss * (2.0f + ss)), ke);
-  st->th = make_float4(t.xh, t.xl, t.eh, t.el);
-  baro_half(I, bx, ke, trw, pe);
-  const float f2 = baro_friction(I, bx, pe);
-  const float e2 = fmaf(ss, f2, ss + f2);
-  st->sig = fmaf(e1, e2, e1 + e2);
-  st->pe_b = pe;
-  npt_geometry(d, I, b, pe);
-}
-
-// Thermostat at the end of the step of parity par, for box b (one thread per
-// box, after the step's kinetic-energy sum is complete): the end half of this
-// step, then the start half of the next one; stores the state after each half
-// and the combined scale S - 1 the next kick1 applies.
+// The same for box b of the step of parity par, from the global sums (one
+// thread per box, in the last block to finish).
 template <bool kNpt>
 __device__ void end_of_step_box(const Dev& d, const Integ& I, int b, int par) {
-  if constexpr (kNpt) {
-    end_of_step_box_npt(d, I, b, par);
-  } else {
-    BoxState* st = d.bst + b;
-    const Box& bx = d.box[b];
-    const double ke0 = __ldcg(&st->ke_acc[par]);
-    ThermoState t = thermo_in(bx, __ldcg(&st->th), ke0);
-    const float se = end_half(I, bx, t);
-    st->th_e = make_float4(t.xh, t.xl, t.eh, t.el);
-    st->ke_last = fma(ke0, (double)(se * (2.0f + se)), ke0);
-    st->s_endc = 1.0 + (double)se;
-    const float ss = start_half(I, bx, t);
-    st->th = make_float4(t.xh, t.xl, t.eh, t.el);
-    st->sig = fmaf(se, ss, se + ss);
-  }
+  BoxState& st = d.bst[b];
+  const double ke0 = __ldcg(&st.ke_acc[par]);
+  const double trw = kNpt ? __ldcg(&st.ew[par][2]) + __ldcg(&st.ew[par][3]) + __ldcg(&st.ew[par][4]) : 0.0;
+  const int r = end_of_step<kNpt, LdGlobal>(I, const_cast<Box*>(d.box)[b], st, ke0, trw);
+  if (r & 2) set_status(d.g, ST_GRID);
+  if (r & 1) d.g->any_rebuild = 1;
 }
 
 // Start half only, from the state after the last end half (a new state, or a
@@ -825,40 +855,45 @@ __device__ __forceinline__ bool block_stop(const Dev& d) {
 // exponent.  Also zeroes f for this step.
 constexpr int kKThreads = 256;  // threads per block of k_kick1 / k_kick2
 
+struct Kick1In {  // one atom's inputs
+  float4 F;
+  uint4 qb;
+  float2 v[3];
+  unsigned long long s[3];
+};
+__device__ __forceinline__ Kick1In kick1_load(const Dev& d, int i) {
+  return {d.f[i], d.qb[i], {d.vx[i], d.vy[i], d.vz[i]}, {d.x[i], d.y[i], d.z[i]}};
+}
+
+// The kick, drift and displacement check of atom i in box b, results stored;
+// moved: the atom is further than the rebuild margin from its list position;
+// lost: a velocity component at or above the runaway threshold, or NaN/inf.
 template <bool kNpt>
-__device__ __forceinline__ void kick1_atom(const Dev& d, const Integ& I, int i, int par, int pend) {
-  // every load first (nothing here is written by another atom's thread);
-  // the fixed-point copy is read only for its box (one box: box 0)
-  const int b = d.nbox == 1 ? 0 : (int)d.q[i].w;
-  const float4 F = d.f[i];
-  const uint4 qb = d.qb[i];
-  const float2 v0[3] = {d.vx[i], d.vy[i], d.vz[i]};
-  const unsigned long long s0[3] = {d.x[i], d.y[i], d.z[i]};
-  const Box& bx = d.box[b];
-  const float sig = d.bst[b].sig;
+__device__ __forceinline__ void kick1_apply(const Dev& d, const Integ& I, const Box& bx, float sig, int i, int b, int pend,
+                                            const Kick1In& in, bool& moved, bool& lost) {
   const float kf = I.cf_f * (pend ? 2.0f + sig : 1.0f);
   const int vexp = bx.vexp_lost;
-  const float Fc[3] = {F.x, F.y, F.z};
-  const uint32_t qbc[3] = {qb.x, qb.y, qb.z};
+  const float Fc[3] = {in.F.x, in.F.y, in.F.z};
+  const uint32_t qbc[3] = {in.qb.x, in.qb.y, in.qb.z};
   float2 vn[3];
   unsigned long long sn[3];
   uint32_t qn[3];
   float dd = 0.f;  // squared displacement since the last build
-  bool lost = false;
+  lost = false;
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     // v + t as hi + lo: two-sum of hi and t, its error added to lo, renormalised
-    const float t = fmaf(sig, v0[c].x, fmaf(sig, v0[c].y, kf * Fc[c]));
-    const float sh = v0[c].x + t;
-    const float bb = sh - v0[c].x;
-    const float er = (v0[c].x - (sh - bb)) + (t - bb);
-    const float lo1 = v0[c].y + er;
+    const float t = fmaf(sig, in.v[c].x, fmaf(sig, in.v[c].y, kf * Fc[c]));
+    const float sh = in.v[c].x + t;
+    const float bb = sh - in.v[c].x;
+    const float er = (in.v[c].x - (sh - bb)) + (t - bb);
+    const float lo1 = in.v[c].y + er;
     const float hi = sh + lo1;
     const float lo = lo1 - (hi - sh);
     const float k64 = bx.dtL64[c];
     const long long inc = f2ll_exact(fmaf(hi, k64, lo * k64));
-    sn[c] = s0[c] + (unsigned long long)inc;
-    if (inc > 0 ? sn[c] < s0[c] : sn[c] > s0[c])  // the 64-bit fraction wrapped: the atom crossed a face
+    sn[c] = in.s[c] + (unsigned long long)inc;
+    if (inc > 0 ? sn[c] < in.s[c] : sn[c] > in.s[c])  // the 64-bit fraction wrapped: the atom crossed a face
       reinterpret_cast<int*>(d.img + i)[c] += inc > 0 ? 1 : -1;
     vn[c] = make_float2(hi, lo);
     qn[c] = q_of(sn[c]);
@@ -875,13 +910,25 @@ __device__ __forceinline__ void kick1_atom(const Dev& d, const Integ& I, int i, 
   d.y[i] = sn[1];
   d.z[i] = sn[2];
   d.q[i] = make_uint4(qn[0], qn[1], qn[2], (unsigned)b);
+  moved = dd > (kNpt ? bx.hs2 : I.half_skin2);
+}
+
+template <bool kNpt>
+__device__ __forceinline__ void kick1_atom(const Dev& d, const Integ& I, int i, int par, int pend) {
+  // every load first (nothing here is written by another atom's thread);
+  // the fixed-point copy is read only for its box (one box: box 0)
+  const int b = d.nbox == 1 ? 0 : (int)d.q[i].w;
+  const Kick1In in = kick1_load(d, i);
+  const Box& bx = d.box[b];
+  bool moved, lost;
+  kick1_apply<kNpt>(d, I, bx, d.bst[b].sig, i, b, pend, in, moved, lost);
   if (i == bx.off) {  // this step's accumulators start from zero
     BoxState* sw = d.bst + b;
     sw->ke_acc[par] = 0.0;
 #pragma unroll
     for (int k2 = 0; k2 < 8; ++k2) sw->ew[par][k2] = 0.0;
   }
-  if (dd > (kNpt ? bx.hs2 : I.half_skin2)) {
+  if (moved) {
     d.bst[b].rebuild = 1;
     d.g->any_rebuild = 1;
   }
@@ -945,11 +992,13 @@ __device__ __forceinline__ int stencil_off(int nc, int o) { return nc >= 3 ? o -
 // fixed-point coordinates are staged and each pair takes its own
 // minimum-image fixed-point difference.
 template <bool kFrame>
-__device__ __forceinline__ void neigh_rows(const Dev& d, const uint4* qa, float4* stg, int a0, int ni, int incl,
-                                           int start, int excl, int total, float L0, float L1, float L2, float rl2) {
+__device__ __forceinline__ bool neigh_rows(const Dev& d, const uint4* qa, float4* stg, int a0, int ni, int incl,
+                                           int start, int excl, int total, float L0, float L1, float L2, float rl2,
+                                           int part, int parts) {
   const int lane = threadIdx.x & 31;
   const unsigned below = (1u << lane) - 1u;  // lanes under this one
   const uint4 o = qa[a0];
+  bool over = false;
   for (int ib = 0; ib < ni; ib += 32) {  // centre atoms of this cell, 32 at a time
     const int nb = min(32, ni - ib);
     const int me = a0 + ib + min(lane, nb - 1);  // lane k's centre
@@ -988,7 +1037,7 @@ __device__ __forceinline__ void neigh_rows(const Dev& d, const uint4* qa, float4
         stg[(bt << 5) + lane] = e;
       }
       __syncwarp();
-      for (int k = 0; k < nb; k += kNeighCentres) {  // kNeighCentres centres over the staged batch (warp-uniform)
+      for (int k = kNeighCentres * part; k < nb; k += kNeighCentres * parts) {  // kNeighCentres centres over the staged batch (warp-uniform)
         float xc[kNeighCentres], yc[kNeighCentres], zc[kNeighCentres];
         int ic[kNeighCentres], cc[kNeighCentres];
         int* rc[kNeighCentres];
@@ -1032,24 +1081,30 @@ __device__ __forceinline__ void neigh_rows(const Dev& d, const uint4* qa, float4
           if (on[c] && lane == k + c) mycount = cc[c];
       }
     }
-    if (lane < nb) d.nbr_cnt[me] = mycount;
+    if (lane < nb && (lane / kNeighCentres) % parts == part) d.nbr_cnt[me] = mycount;
     // the longest row: one atomic per warp, and none once the running maximum
     // covers it (rather than one per centre on this one word)
     const int wmax = __reduce_max_sync(kFull, lane < nb ? mycount : 0);
+    over |= wmax > d.W;
     if (lane == 0 && wmax > *(volatile int*)&d.g->max_count) {
       atomicMax(&d.g->max_count, wmax);
       if (wmax > d.W) set_status(d.g, ST_OVERFLOW);
     }
   }
+  return over;
 }
 
-// stg: the warp's kNStage float4 of shared memory.
-__device__ void neigh_cell_warp(const Dev& d, const uint4* qa, float4* stg, int c, float rl2) {
+// The rows of cell c of the box bx; stg: the warp's kNStage float4 of shared
+// memory.  A cell may be shared by `parts` warps, each staging the stencil
+// for itself and taking every parts-th group of kNeighCentres centres (a
+// build with fewer cells than warps is as long as one cell's chain of
+// dependent batches).  Returns whether a row was wider than its allocation.
+__device__ bool neigh_cell(const Dev& d, const Box& bx, const uint4* qa, float4* stg, int c, float rl2, int part = 0,
+                           int parts = 1) {
   const int lane = threadIdx.x & 31;
   const int a0 = d.cell_start[c];
   const int ni = d.cell_start[c + 1] - a0;
-  if (ni == 0 || !box_flagged(d, d.cell_box[c])) return;  // warp-uniform
-  const Box& bx = d.box[d.cell_box[c]];
+  if (ni <= kNeighCentres * part) return false;  // warp-uniform
   const int cl = c - bx.cell_off;
   const int cx = cl % bx.nc[0], cy = (cl / bx.nc[0]) % bx.nc[1], cz = cl / (bx.nc[0] * bx.nc[1]);
   const bool frame = bx.nc[0] >= 4 && bx.nc[1] >= 4 && bx.nc[2] >= 4;  // warp-uniform
@@ -1087,10 +1142,13 @@ __device__ void neigh_cell_warp(const Dev& d, const uint4* qa, float4* stg, int 
   const int excl = incl - cnt;
   const int total = __shfl_sync(kFull, incl, 31);
   const float L0 = bx.Lq[0], L1 = bx.Lq[1], L2 = bx.Lq[2];
-  if (frame)
-    neigh_rows<true>(d, qa, stg, a0, ni, incl, start, excl, total, L0, L1, L2, rl2);
-  else
-    neigh_rows<false>(d, qa, stg, a0, ni, incl, start, excl, total, L0, L1, L2, rl2);
+  return frame ? neigh_rows<true>(d, qa, stg, a0, ni, incl, start, excl, total, L0, L1, L2, rl2, part, parts)
+               : neigh_rows<false>(d, qa, stg, a0, ni, incl, start, excl, total, L0, L1, L2, rl2, part, parts);
+}
+
+__device__ __forceinline__ void neigh_cell_warp(const Dev& d, const uint4* qa, float4* stg, int c, float rl2) {
+  const int b = d.cell_box[c];
+  if (box_flagged(d, b)) neigh_cell(d, d.box[b], qa, stg, c, rl2);  // warp-uniform
 }
 
 // ---------------------------------------------------------------------------
@@ -1327,19 +1385,20 @@ __device__ __noinline__ int species_item(const Dev& d, const SpPair* sp, const f
 // with the leg reversed), so no leg force is scattered; centres over the
 // staged-leg limit keep the scatter path (pass 1), and their neighbours add
 // their own terms' forces to them by scatter.
-template <bool kCount, int kSp = 0, int KG = kG, int kOwn = 0>
-__device__ void force_block(const Dev& d, const FParams& P,
-                            LegTableT<(kSp ? kLMaxSp : kLMax), kFThreads / KG>& T, int blk, int par,
-                            const SpPair* sps = nullptr, int nsp = 1, const float2* stt = nullptr) {
+// force_group: the 32 / KG centres of one warp (centre i of this lane's
+// group; valid: there is one), ue and aux the warp's rows of the leg table;
+// adds to acc (E2, E3, W xx yy zz xy xz yz) and returns the centre's box.
+// Synchronises the warp only.
+template <bool kCount, int kSp, int KG, int kOwn>
+__device__ __forceinline__ int force_group(const Dev& d, const FParams& P, float4* ue, float4* aux, int i, bool valid, int par,
+                                           float (&acc)[8], const SpPair* sps = nullptr, int nsp = 1,
+                                           const float2* stt = nullptr) {
   constexpr int kLM = kSp ? kLMaxSp : kLMax;  // legs staged per centre
   const int lane = threadIdx.x & 31;
   const int g = threadIdx.x & (KG - 1);
-  const int a = threadIdx.x / KG;
+  const int a = lane / KG;
   const int sw = (a * KG) & 7;                                  // the row's bank-group swizzle
   auto at = [&](int l) { return a * kLM + (l ^ sw); };          // leg l of this centre
-  const int i = blk * (kFThreads / KG) + a;
-  const bool valid = i < d.N;
-  float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};  // E2, E3, W xx yy zz xy xz yz
   float fx = 0.f, fy = 0.f, fz = 0.f;  // force on the centre (pair part and three-body reaction)
   uint4 qi = make_uint4(0u, 0u, 0u, 0u);
   int cnt = 0, b = -1;
@@ -1371,10 +1430,10 @@ __device__ void force_block(const Dev& d, const FParams& P,
       const int j = d.legs[(size_t)i * kLMax + l];
       const uint4 qj = d.q[j];
       const float dx = fix_diff(qi.x, qj.x, L0), dy = fix_diff(qi.y, qj.y, L1), dz = fix_diff(qi.z, qj.z, L2);
-      T.ue[at(l)] = make_float4(dx, dy, dz, __int_as_float(j));
+      ue[at(l)] = make_float4(dx, dy, dz, __int_as_float(j));
     }
   } else if constexpr (kSp == 0) {
-    nl = stage_legs<KG, kLM>(d, P.rc2, T.ue, at, qi, L0, L1, L2, row, cnt);
+    nl = stage_legs<KG, kLM>(d, P.rc2, ue, at, qi, L0, L1, L2, row, cnt);
   } else {
     const int iters = __reduce_max_sync(kFull, (cnt + KG - 1) / KG);
     const unsigned gsh = lane & ~(KG - 1);
@@ -1413,8 +1472,8 @@ __device__ void force_block(const Dev& d, const FParams& P,
         const unsigned m = (__ballot_sync(kFull, hit) >> gsh) & ((1u << KG) - 1u);
         const int pos = nl + __popc(m & ((1u << g) - 1u));
         if (hit && pos < kLM) {  // (the pair's cutoff test needs r^2 again in phase B: kept)
-          T.ue[at(pos)] = make_float4(dx, dy, dz, r2);
-          T.aux[at(pos)] = make_float4(__int_as_float(tj[t]), 0.f, 0.f, __int_as_float(jr[t]));
+          ue[at(pos)] = make_float4(dx, dy, dz, r2);
+          aux[at(pos)] = make_float4(__int_as_float(tj[t]), 0.f, 0.f, __int_as_float(jr[t]));
         }
         nl += __popc(m);
       }
@@ -1422,7 +1481,7 @@ __device__ void force_block(const Dev& d, const FParams& P,
   }
   __syncwarp();
   if constexpr (kOwn == 1) {  // the staged legs for pass 2
-    for (int l = g; l < min(nl, kLM); l += KG) d.legs[(size_t)i * kLMax + l] = __float_as_int(T.ue[at(l)].w);
+    for (int l = g; l < min(nl, kLM); l += KG) d.legs[(size_t)i * kLMax + l] = __float_as_int(ue[at(l)].w);
     if (valid && g == 0) d.nleg[i] = nl <= kLM ? nl : -1;
   }
   // ---- leg phase B: leg terms for the compacted legs only, spread over the
@@ -1433,8 +1492,8 @@ __device__ void force_block(const Dev& d, const FParams& P,
   float mxx = 0.f, myy = 0.f, mzz = 0.f, mxy = 0.f, mxz = 0.f, myz = 0.f;     // M
   int nvalid = 0;  // legs inside their own pair's cutoff (kSp counting)
   for (int l = g; l < nstage; l += KG) {
-    float4* ue_p = T.ue + at(l);
-    float4* ax_p = T.aux + at(l);
+    float4* ue_p = ue + at(l);
+    float4* ax_p = aux + at(l);
     const float4 rec = *ue_p;
     // (one species: the record is d and j; r^2 as in phase A's test)
     const float r2 = kSp ? rec.w : fmaf(rec.x, rec.x, fmaf(rec.y, rec.y, rec.z * rec.z));
@@ -1530,8 +1589,8 @@ __device__ void force_block(const Dev& d, const FParams& P,
     // ---- leg phase C (any table): leg j against every other leg k
     const float2* stc = stt + ti * nsp * nsp;
     for (int l = g; l < nstage; l += KG) {
-      const float4 uj = T.ue[at(l)];
-      const float4 xj = T.aux[at(l)];
+      const float4 uj = ue[at(l)];
+      const float4 xj = aux[at(l)];
       if (uj.w == 0.f) continue;  // leg dropped in phase B
       const int wj = __float_as_int(xj.w);
       const float2* stj = stc + (wj >> 28) * nsp;
@@ -1540,9 +1599,9 @@ __device__ void force_block(const Dev& d, const FParams& P,
       const float nde = xj.y;
       float gx = 0.f, gy = 0.f, gz = 0.f;  // three-body force on the partner of leg j
       for (int k = 0; k < nstage; ++k) {
-        const float4 uk = T.ue[at(k)];
+        const float4 uk = ue[at(k)];
         if (k == l || uk.w == 0.f) continue;
-        const float2 lc = stj[__float_as_int(T.aux[at(k)].w) >> 28];  // (lambda eps, cos theta0)
+        const float2 lc = stj[__float_as_int(aux[at(k)].w) >> 28];  // (lambda eps, cos theta0)
         const float c = fmaf(uj.x, uk.x, fmaf(uj.y, uk.y, uj.z * uk.z));
         const float D = c - lc.y;
         const float gg = lc.x * uj.w * uk.w * D;
@@ -1600,8 +1659,8 @@ __device__ void force_block(const Dev& d, const FParams& P,
     return Cj;
   };
   for (int l = g; l < nstage; l += KG) {
-    const float4 uj = T.ue[at(l)];
-    const float4 xj = T.aux[at(l)];
+    const float4 uj = ue[at(l)];
+    const float4 xj = aux[at(l)];
     const float ee = uj.w;
     if (ee == 0.f) continue;  // leg dropped in phase B
     const float r = xj.z;
@@ -1678,6 +1737,19 @@ __device__ void force_block(const Dev& d, const FParams& P,
       atomicAdd((unsigned long long*)&d.g->ntrip, tri);
     }
   }
+  return b;
+}
+
+// One block of kFThreads / KG centres; every thread of the block calls it.
+template <bool kCount, int kSp = 0, int KG = kG, int kOwn = 0>
+__device__ void force_block(const Dev& d, const FParams& P,
+                            LegTableT<(kSp ? kLMaxSp : kLMax), kFThreads / KG>& T, int blk, int par,
+                            const SpPair* sps = nullptr, int nsp = 1, const float2* stt = nullptr) {
+  constexpr int kRows = (32 / KG) * (kSp ? kLMaxSp : kLMax);  // records of a warp's centres
+  float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  const int w = (int)(threadIdx.x >> 5);
+  const int i = blk * (kFThreads / KG) + (int)threadIdx.x / KG;
+  const int b = force_group<kCount, kSp, KG, kOwn>(d, P, T.ue + w * kRows, T.aux + w * kRows, i, i < d.N, par, acc, sps, nsp, stt);
   box_accumulate<8>(acc, b, [&](int bb) { return &d.bst[bb].ew[par][0]; });
 }
 
