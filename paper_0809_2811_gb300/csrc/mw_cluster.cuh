@@ -181,7 +181,7 @@ __device__ __forceinline__ bool clu_rebuild(const Dev& d, CluShared& S, float4* 
   for (int k = (int)rank * T + tid; k < ncb; k += (int)size * T) d.cell_cnt[bx.cell_off + k] = 0;
   bool over = false;
   float4* stg = tab + wid * (kCluWarpBytes / (int)sizeof(float4));
-  static_assert(kCluWarpBytes >= kNStage * (int)sizeof(float4), "staging slices");
+  static_assert(kCluWarpBytes >= kNSlice * (int)sizeof(float4), "staging slices");
   const int nw = (T >> 5) * (int)size;
   const int parts = max(1, min(4, nw / ncb));
   for (int k = wid * (int)size + (int)rank; k < ncb * parts; k += nw)

@@ -249,13 +249,6 @@ __device__ __forceinline__ float fix_diff(uint32_t a, uint32_t b, float lq) {  /
   return __int2float_rn((int)(b - a)) * lq;
 }
 
-// Store of v to *addr when p holds, as one predicated store (no branch
-// around it).
-__device__ __forceinline__ void st_if(bool p, int* addr, int v) {
-  asm volatile("{\n .reg .pred q;\n setp.ne.b32 q, %0, 0;\n @q st.global.b32 [%1], %2;\n}" ::"r"((int)p), "l"(addr), "r"(v)
-               : "memory");
-}
-
 __device__ __forceinline__ void red_add_v4(float4* addr, float a, float b, float c) {
   asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(addr), "f"(a), "f"(b), "f"(c), "f"(0.0f)
                : "memory");
@@ -963,52 +956,222 @@ __device__ __forceinline__ float kick2_atom(const Dev& d, const Integ& I, int i,
 }
 
 // ---------------------------------------------------------------------------
-// Neighbour list (a3): one warp per cell.  The candidates of the
-// (deduplicated) 27-cell stencil are flattened in stencil order and staged,
-// up to kNStage at a time, in the warp's slice of shared memory; then the
-// centre atoms of the cell, kNeighCentres at a time, run over the staged
-// candidates 32 at a time (one per lane), and the hits of each batch go
-// straight to their places in each centre's row (its running count plus the
-// hits of lower lanes), so each row lists its neighbours in stencil order.
+// Neighbour list (a3): one warp per cell.  The candidates of the stencil are
+// staged, up to kNStage at a time, in the warp's slice of shared memory; then
+// the centre atoms of the cell, kNeighCentres at a time, run over the staged
+// candidates, and the hits of each batch go straight to their places in each
+// centre's row (its running count plus the hits of lower lanes).  Bound by
+// instruction issue.  Two forms:
+//   neigh_rows_frame: every axis of the box has at least 4 cells;
+//   neigh_rows_wrap: grids of 1-3 cells on an axis, where the stencil wraps
+//     round the box: the (deduplicated) cells' fixed-point coordinates are
+//     staged and each pair takes its own minimum-image difference.
 constexpr int kNStage = 256;  // candidates staged per warp at a time (4 KB)
+constexpr int kNSlice = kNStage + 8;  // float4 of shared memory a warp: the candidates, a mark per candidate, 18 runs
 constexpr int kNeighCentres = 2;  // centres tested together against each staged batch
 __device__ __forceinline__ int stencil_n(int nc) { return nc >= 3 ? 3 : nc; }
 __device__ __forceinline__ int stencil_off(int nc, int o) { return nc >= 3 ? o - 1 : o; }
 
-// The rows of one cell's centres (neigh_cell_warp).  Staging: lane t of a
-// batch takes candidate t of the stencil's concatenated cells (located by a
-// binary search over the warp's inclusive counts) and stores (x, y, z, j);
-// entries past the last candidate get j = -1 (and, with kFrame, an offset
-// no distance test passes).  The centres go over a batch kNeighCentres at a
-// time, so that each staged record is read once for all of them (2 measured
-// fastest against 1, 3 and 4).  A count past the row
-// width (an overflow: the status makes the caller grow the rows and build
-// again) writes to the row's last slot, never past it.
-// kFrame: every axis of the box has at least 4 cells, so each candidate lies
-// within two cell edges of o, the cell's first atom; offsets from o are exact
-// fixed-point differences with no wrap, converted once per atom and staged
-// as FP32, and a pair's displacement is their FP32 difference.  Otherwise
-// (grids of 1-3 cells on an axis, where the stencil wraps round the box) the
-// fixed-point coordinates are staged and each pair takes its own
-// minimum-image fixed-point difference.
-template <bool kFrame>
-__device__ __forceinline__ bool neigh_rows(const Dev& d, const uint4* qa, float4* stg, int a0, int ni, int incl,
-                                           int start, int excl, int total, float L0, float L1, float L2, float rl2,
-                                           int part, int parts) {
+// Two FP32 values in a register pair: the packed instructions round each half
+// as the scalar ones do, at one issue slot for both.
+__device__ __forceinline__ unsigned long long pk2(float a, float b) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void upk2(unsigned long long v, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b) {
+  unsigned long long r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigned long long b) {
+  unsigned long long r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
+  unsigned long long r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
+// One candidate per lane against one centre: its hit (r2 < rl2, not the centre
+// itself) is stored as j at row[min(count + hits of lower lanes, last)], and
+// the count of the warp's hits is added to count.  In one piece, so that the
+// hit stays a predicate from the test to the store.
+__device__ __forceinline__ void neigh_hit(float r2, float rl2, int j, int centre, unsigned below, int last, int* row, int& count) {
+  asm volatile(
+      "{\n .reg .pred p;\n .reg .b32 m, t;\n .reg .b64 a;\n"
+      " setp.ne.s32 p, %2, %3;\n"
+      " setp.lt.and.f32 p, %1, %4, p;\n"
+      " vote.sync.ballot.b32 m, p, 0xffffffff;\n"
+      " and.b32 t, m, %5;\n"
+      " popc.b32 t, t;\n"
+      " add.s32 t, t, %0;\n"
+      " min.s32 t, t, %6;\n"
+      " mad.wide.s32 a, t, 4, %7;\n"
+      " @p st.global.b32 [a], %2;\n"
+      " popc.b32 t, m;\n"
+      " add.s32 %0, %0, t;\n}"
+      : "+r"(count)
+      : "f"(r2), "r"(j), "r"(centre), "f"(rl2), "r"(below), "r"(last), "l"(row)
+      : "memory");
+}
+
+// The longest row so far, from one warp's rows: one atomic per warp, and none
+// once the running maximum covers it (rather than one per centre on this one
+// word).  Returns whether a row is wider than its allocation.
+__device__ __forceinline__ bool neigh_count(const Dev& d, int mycount) {
+  const int wmax = __reduce_max_sync(kFull, mycount);
+  if ((threadIdx.x & 31) == 0 && wmax > *(volatile int*)&d.g->max_count) {
+    atomicMax(&d.g->max_count, wmax);
+    if (wmax > d.W) set_status(d.g, ST_OVERFLOW);
+  }
+  return wmax > d.W;
+}
+
+// The rows of one cell's centres, every axis of the box at least 4 cells long:
+// each candidate then lies within two cell edges of o, the cell's first atom;
+// offsets from o are exact fixed-point differences with no wrap, converted
+// once per atom and staged as FP32, and a pair's displacement is their FP32
+// difference.  The stencil is 9 runs of atoms (three cells along x lie next
+// to one another; a cell at the box's x face splits each run in two): lane r
+// holds run r, first its first atom, excl its place among the candidates.
+// Each lane tests two neighbouring candidates at a time with packed FP32
+// arithmetic, against kNeighCentres centres per staged record read.  Padding
+// entries fail the test by their offset.  A count past the row width (an
+// overflow: the status makes the caller grow the rows and build again) writes
+// to the row's last slot, never past it.
+// 2^20-atom slab, full build: 277 us, 253 M warp instructions (310 us and 289 M with one candidate a lane and every staging
+// batch located by a binary search over the 27 cells; 3 centres at a time 290 us).
+__device__ __forceinline__ bool neigh_rows_frame(const Dev& d, const uint4* qa, const uint4& o, float* stg, int a0, int ni, int first, int cnt,
+                                                 int excl, int total, float L0, float L1, float L2, float rl2, int part,
+                                                 int parts) {
+  static_assert(kNStage % 64 == 0, "whole groups of two candidates a lane");
   const int lane = threadIdx.x & 31;
   const unsigned below = (1u << lane) - 1u;  // lanes under this one
-  const uint4 o = qa[a0];
+  float* const sx = stg;
+  float* const sy = stg + kNStage;
+  float* const sz = stg + 2 * kNStage;
+  int* const sj = reinterpret_cast<int*>(stg + 3 * kNStage);
+  unsigned* const marks = reinterpret_cast<unsigned*>(stg + 4 * kNStage);
+  int* const delta = reinterpret_cast<int*>(marks + kNStage / 32);  // per run that is not empty: first atom - place
+  bool over = false;
+  {
+    const unsigned full = __ballot_sync(kFull, cnt > 0);
+    if (cnt > 0) delta[__popc(full & below)] = first - excl;
+  }
+  for (int ib = 0; ib < ni; ib += 32) {  // centre atoms of this cell, 32 at a time
+    const int nb = min(32, ni - ib);
+    const uint4 qmine = qa[a0 + ib + min(lane, nb - 1)];  // lane k's centre
+    const float cx = fix_diff(qmine.x, o.x, L0), cy = fix_diff(qmine.y, o.y, L1), cz = fix_diff(qmine.z, o.z, L2);  // o - centre
+    int mycount = 0;  // neighbours of lane k's centre so far
+    for (int c0 = 0; c0 < total; c0 += kNStage) {  // chunks of the candidate list (warp-uniform)
+      const int nch = min(kNStage, total - c0);
+      const int nbat = (nch + 31) >> 5, ngrp = nbat >> 1;  // whole groups of 64; an odd batch of 32 is left over
+      __syncwarp();  // the previous chunk's readers are done
+      // the run that holds candidate t: as many marks (first candidates of
+      // runs that are not empty) up to t, counted from the runs before c0
+      if (lane < kNStage / 32) marks[lane] = 0u;
+      __syncwarp();
+      if (cnt > 0 && excl >= c0 && excl < c0 + kNStage) atomicOr(marks + ((excl - c0) >> 5), 1u << ((excl - c0) & 31));
+      int seen = __popc(__ballot_sync(kFull, cnt > 0 && excl < c0)) - 1;
+      __syncwarp();
+      for (int t = lane; t - lane < nch; t += 32) {  // (warp-uniform)
+        const unsigned mk = marks[t >> 5];
+        const int r = seen + __popc(mk & (below | (1u << lane)));
+        seen += __popc(mk);
+        float x = 1e30f, y = 0.f, z = 0.f;  // past the last candidate: no hit
+        int j = -1;
+        if (t < nch) {
+          j = c0 + t + delta[r];
+          const uint4 qj = qa[j];
+          x = fix_diff(o.x, qj.x, L0);
+          y = fix_diff(o.y, qj.y, L1);
+          z = fix_diff(o.z, qj.z, L2);
+        }
+        sx[t] = x;
+        sy[t] = y;
+        sz[t] = z;
+        sj[t] = j;
+      }
+      __syncwarp();
+      for (int k = kNeighCentres * part; k < nb; k += kNeighCentres * parts) {  // (warp-uniform)
+        unsigned long long xc[kNeighCentres], yc[kNeighCentres], zc[kNeighCentres];
+        int ic[kNeighCentres], cc[kNeighCentres];
+        int* rc[kNeighCentres];
+        bool on[kNeighCentres];  // (a last group may hold fewer centres)
+        const int wl = d.W - 1;
+#pragma unroll
+        for (int c = 0; c < kNeighCentres; ++c) {
+          on[c] = k + c < nb;
+          const int kc = on[c] ? k + c : k;
+          float x = __shfl_sync(kFull, cx, kc);
+          const float y = __shfl_sync(kFull, cy, kc), z = __shfl_sync(kFull, cz, kc);
+          if (!on[c]) x = 1e30f;  // no hits
+          xc[c] = pk2(x, x);
+          yc[c] = pk2(y, y);
+          zc[c] = pk2(z, z);
+          ic[c] = a0 + ib + kc;
+          cc[c] = __shfl_sync(kFull, mycount, kc);
+          rc[c] = d.nbr + (size_t)(a0 + ib + kc) * d.W;
+        }
+        for (int gr = 0; gr < ngrp; ++gr) {
+          const int at = (gr << 6) + 2 * lane;
+          const unsigned long long ex = *reinterpret_cast<const unsigned long long*>(sx + at);
+          const unsigned long long ey = *reinterpret_cast<const unsigned long long*>(sy + at);
+          const unsigned long long ez = *reinterpret_cast<const unsigned long long*>(sz + at);
+          const int2 j = *reinterpret_cast<const int2*>(sj + at);
+#pragma unroll
+          for (int c = 0; c < kNeighCentres; ++c) {
+            const unsigned long long dx = add2(ex, xc[c]), dy = add2(ey, yc[c]), dz = add2(ez, zc[c]);
+            float r0, r1;
+            upk2(fma2(dx, dx, fma2(dy, dy, mul2(dz, dz))), r0, r1);
+            neigh_hit(r0, rl2, j.x, ic[c], below, wl, rc[c], cc[c]);
+            neigh_hit(r1, rl2, j.y, ic[c], below, wl, rc[c], cc[c]);
+          }
+        }
+        if (nbat & 1) {  // one candidate a lane
+          const int at = (ngrp << 6) + lane;
+          const float ex = sx[at], ey = sy[at], ez = sz[at];
+          const int j = sj[at];
+#pragma unroll
+          for (int c = 0; c < kNeighCentres; ++c) {
+            float xx, yy, zz, u;
+            upk2(xc[c], xx, u);
+            upk2(yc[c], yy, u);
+            upk2(zc[c], zz, u);
+            const float dx = ex + xx, dy = ey + yy, dz = ez + zz;
+            neigh_hit(fmaf(dx, dx, fmaf(dy, dy, dz * dz)), rl2, j, ic[c], below, wl, rc[c], cc[c]);
+          }
+        }
+#pragma unroll
+        for (int c = 0; c < kNeighCentres; ++c)
+          if (on[c] && lane == k + c) mycount = cc[c];
+      }
+    }
+    if (lane < nb && (lane / kNeighCentres) % parts == part) d.nbr_cnt[a0 + ib + lane] = mycount;
+    over |= neigh_count(d, mycount);
+  }
+  return over;
+}
+
+// The same for grids of 1-3 cells on an axis.  Staging: lane t of a batch
+// takes candidate t of the stencil's concatenated cells (located by a binary
+// search over the warp's inclusive counts) and stores (x, y, z, j), x, y, z
+// fixed-point; entries past the last candidate get j = -1.
+__device__ __forceinline__ bool neigh_rows_wrap(const Dev& d, const uint4* qa, float4* stg, int a0, int ni, int incl, int start,
+                                                int excl, int total, float L0, float L1, float L2, float rl2, int part,
+                                                int parts) {
+  const int lane = threadIdx.x & 31;
+  const unsigned below = (1u << lane) - 1u;  // lanes under this one
   bool over = false;
   for (int ib = 0; ib < ni; ib += 32) {  // centre atoms of this cell, 32 at a time
     const int nb = min(32, ni - ib);
-    const int me = a0 + ib + min(lane, nb - 1);  // lane k's centre
-    const uint4 qmine = qa[me];
-    float cx, cy, cz;  // its offset from o (kFrame) or its fixed-point position
-    if constexpr (kFrame) {
-      cx = fix_diff(o.x, qmine.x, L0); cy = fix_diff(o.y, qmine.y, L1); cz = fix_diff(o.z, qmine.z, L2);
-    } else {
-      cx = __uint_as_float(qmine.x); cy = __uint_as_float(qmine.y); cz = __uint_as_float(qmine.z);
-    }
+    const uint4 qmine = qa[a0 + ib + min(lane, nb - 1)];  // lane k's centre
     int mycount = 0;  // neighbours of lane k's centre so far
     for (int c0 = 0; c0 < total; c0 += kNStage) {  // chunks of the candidate list (warp-uniform)
       const int nch = min(kNStage, total - c0);
@@ -1025,76 +1188,39 @@ __device__ __forceinline__ bool neigh_rows(const Dev& d, const uint4* qa, float4
         }
         const int sk = __shfl_sync(kFull, start, lo);
         const int ek = __shfl_sync(kFull, excl, lo);
-        float4 e = make_float4(kFrame ? 1e30f : 0.f, 0.f, 0.f, __int_as_float(-1));
+        float4 e = make_float4(0.f, 0.f, 0.f, __int_as_float(-1));
         if (t < total) {
           const int j = sk + (t - ek);
           const uint4 qj = qa[j];
-          if constexpr (kFrame)
-            e = make_float4(fix_diff(o.x, qj.x, L0), fix_diff(o.y, qj.y, L1), fix_diff(o.z, qj.z, L2), __int_as_float(j));
-          else
-            e = make_float4(__uint_as_float(qj.x), __uint_as_float(qj.y), __uint_as_float(qj.z), __int_as_float(j));
+          e = make_float4(__uint_as_float(qj.x), __uint_as_float(qj.y), __uint_as_float(qj.z), __int_as_float(j));
         }
         stg[(bt << 5) + lane] = e;
       }
       __syncwarp();
-      for (int k = kNeighCentres * part; k < nb; k += kNeighCentres * parts) {  // kNeighCentres centres over the staged batch (warp-uniform)
-        float xc[kNeighCentres], yc[kNeighCentres], zc[kNeighCentres];
-        int ic[kNeighCentres], cc[kNeighCentres];
-        int* rc[kNeighCentres];
-        bool on[kNeighCentres];  // (a last group may hold fewer centres)
-        const int wl = d.W - 1;
-#pragma unroll
-        for (int c = 0; c < kNeighCentres; ++c) {
-          on[c] = k + c < nb;
-          const int kc = on[c] ? k + c : k;
-          xc[c] = __shfl_sync(kFull, cx, kc);
-          yc[c] = __shfl_sync(kFull, cy, kc);
-          zc[c] = __shfl_sync(kFull, cz, kc);
-          ic[c] = a0 + ib + kc;
-          cc[c] = __shfl_sync(kFull, mycount, kc);
-          rc[c] = d.nbr + (size_t)ic[c] * d.W;
-        }
-#pragma unroll 2
+      for (int k = 0; k < nb; ++k) {  // one centre over the staged batch (warp-uniform)
+        if ((k / kNeighCentres) % parts != part) continue;
+        const uint32_t xc = __shfl_sync(kFull, qmine.x, k), yc = __shfl_sync(kFull, qmine.y, k), zc = __shfl_sync(kFull, qmine.z, k);
+        int cc = __shfl_sync(kFull, mycount, k);
+        const int ic = a0 + ib + k;
+        int* const rc = d.nbr + (size_t)ic * d.W;
         for (int bt = 0; bt < nbat; ++bt) {
           const float4 e = stg[(bt << 5) + lane];
           const int j = __float_as_int(e.w);
-          // (kFrame: padding entries fail the distance test by their offset)
-          const bool live = kFrame || j >= 0;
-#pragma unroll
-          for (int c = 0; c < kNeighCentres; ++c) {
-            float dx, dy, dz;
-            if constexpr (kFrame) {
-              dx = e.x - xc[c]; dy = e.y - yc[c]; dz = e.z - zc[c];
-            } else {
-              dx = fix_diff(__float_as_uint(xc[c]), __float_as_uint(e.x), L0);
-              dy = fix_diff(__float_as_uint(yc[c]), __float_as_uint(e.y), L1);
-              dz = fix_diff(__float_as_uint(zc[c]), __float_as_uint(e.z), L2);
-            }
-            const bool p = (c == 0 || on[c]) && live && j != ic[c] && fmaf(dx, dx, fmaf(dy, dy, dz * dz)) < rl2;
-            const unsigned bm = __ballot_sync(kFull, p);
-            st_if(p, rc[c] + min(cc[c] + __popc(bm & below), wl), j);
-            cc[c] += __popc(bm);
-          }
+          const float dx = fix_diff(xc, __float_as_uint(e.x), L0), dy = fix_diff(yc, __float_as_uint(e.y), L1),
+                      dz = fix_diff(zc, __float_as_uint(e.z), L2);
+          const float r2 = j >= 0 ? fmaf(dx, dx, fmaf(dy, dy, dz * dz)) : 1e30f;
+          neigh_hit(r2, rl2, j, ic, below, d.W - 1, rc, cc);
         }
-#pragma unroll
-        for (int c = 0; c < kNeighCentres; ++c)
-          if (on[c] && lane == k + c) mycount = cc[c];
+        if (lane == k) mycount = cc;
       }
     }
-    if (lane < nb && (lane / kNeighCentres) % parts == part) d.nbr_cnt[me] = mycount;
-    // the longest row: one atomic per warp, and none once the running maximum
-    // covers it (rather than one per centre on this one word)
-    const int wmax = __reduce_max_sync(kFull, lane < nb ? mycount : 0);
-    over |= wmax > d.W;
-    if (lane == 0 && wmax > *(volatile int*)&d.g->max_count) {
-      atomicMax(&d.g->max_count, wmax);
-      if (wmax > d.W) set_status(d.g, ST_OVERFLOW);
-    }
+    if (lane < nb && (lane / kNeighCentres) % parts == part) d.nbr_cnt[a0 + ib + lane] = mycount;
+    over |= neigh_count(d, mycount);
   }
   return over;
 }
 
-// The rows of cell c of the box bx; stg: the warp's kNStage float4 of shared
+// The rows of cell c of the box bx; stg: the warp's kNSlice float4 of shared
 // memory.  A cell may be shared by `parts` warps, each staging the stencil
 // for itself and taking every parts-th group of kNeighCentres centres (a
 // build with fewer cells than warps is as long as one cell's chain of
@@ -1105,33 +1231,40 @@ __device__ bool neigh_cell(const Dev& d, const Box& bx, const uint4* qa, float4*
   const int a0 = d.cell_start[c];
   const int ni = d.cell_start[c + 1] - a0;
   if (ni <= kNeighCentres * part) return false;  // warp-uniform
-  const int cl = c - bx.cell_off;
-  const int cx = cl % bx.nc[0], cy = (cl / bx.nc[0]) % bx.nc[1], cz = cl / (bx.nc[0] * bx.nc[1]);
+  // the cell's coordinates from its first atom, by the rule that binned it
+  // (three high products instead of three integer divisions)
+  const uint4 o = qa[a0];
+  const int cx = (int)__umulhi(o.x, (unsigned)bx.nc[0]), cy = (int)__umulhi(o.y, (unsigned)bx.nc[1]),
+            cz = (int)__umulhi(o.z, (unsigned)bx.nc[2]);
   const bool frame = bx.nc[0] >= 4 && bx.nc[1] >= 4 && bx.nc[2] >= 4;  // warp-uniform
+  const float L0 = bx.Lq[0], L1 = bx.Lq[1], L2 = bx.Lq[2];
   int start = 0, cnt = 0;
-  int X = -1, Y = 0, Z = 0;  // lane's stencil cell
-  if (frame) {  // 3 x 3 x 3 distinct cells; offsets -1, 0, 1 wrap by one compare
-    if (lane < 27) {
-      X = cx + lane % 3 - 1;
-      Y = cy + (lane / 3) % 3 - 1;
-      Z = cz + lane / 9 - 1;
-      X += X < 0 ? bx.nc[0] : (X >= bx.nc[0] ? -bx.nc[0] : 0);
+  if (frame) {  // lanes 0-8: the runs of three x cells (two at an x face); lanes 9-17: the cell round the face
+    const int r = lane < 9 ? lane : lane - 9;
+    if (lane < 18) {
+      int Y = cy + r % 3 - 1, Z = cz + r / 3 - 1;
       Y += Y < 0 ? bx.nc[1] : (Y >= bx.nc[1] ? -bx.nc[1] : 0);
       Z += Z < 0 ? bx.nc[2] : (Z >= bx.nc[2] ? -bx.nc[2] : 0);
+      const int row = bx.cell_off + bx.nc[0] * (Y + bx.nc[1] * Z);
+      int c0 = max(cx - 1, 0), c1 = min(cx + 2, bx.nc[0]);
+      if (lane >= 9) {
+        c0 = cx == 0 ? bx.nc[0] - 1 : 0;
+        c1 = cx == 0 ? bx.nc[0] : (cx == bx.nc[0] - 1 ? 1 : 0);
+      }
+      start = d.cell_start[row + c0];
+      cnt = d.cell_start[row + c1] - start;
     }
   } else {
     const int nx = stencil_n(bx.nc[0]), ny = stencil_n(bx.nc[1]), nz = stencil_n(bx.nc[2]);
     if (lane < nx * ny * nz) {
       const int ox = lane % nx, oy = (lane / nx) % ny, oz = lane / (nx * ny);
-      X = (cx + stencil_off(bx.nc[0], ox) + bx.nc[0]) % bx.nc[0];
-      Y = (cy + stencil_off(bx.nc[1], oy) + bx.nc[1]) % bx.nc[1];
-      Z = (cz + stencil_off(bx.nc[2], oz) + bx.nc[2]) % bx.nc[2];
+      const int X = (cx + stencil_off(bx.nc[0], ox) + bx.nc[0]) % bx.nc[0];
+      const int Y = (cy + stencil_off(bx.nc[1], oy) + bx.nc[1]) % bx.nc[1];
+      const int Z = (cz + stencil_off(bx.nc[2], oz) + bx.nc[2]) % bx.nc[2];
+      const int cc = bx.cell_off + X + bx.nc[0] * (Y + bx.nc[1] * Z);
+      start = d.cell_start[cc];
+      cnt = d.cell_start[cc + 1] - start;
     }
-  }
-  if (X >= 0) {
-    const int cc = bx.cell_off + X + bx.nc[0] * (Y + bx.nc[1] * Z);
-    start = d.cell_start[cc];
-    cnt = d.cell_start[cc + 1] - start;
   }
   int incl = cnt;
 #pragma unroll
@@ -1141,9 +1274,10 @@ __device__ bool neigh_cell(const Dev& d, const Box& bx, const uint4* qa, float4*
   }
   const int excl = incl - cnt;
   const int total = __shfl_sync(kFull, incl, 31);
-  const float L0 = bx.Lq[0], L1 = bx.Lq[1], L2 = bx.Lq[2];
-  return frame ? neigh_rows<true>(d, qa, stg, a0, ni, incl, start, excl, total, L0, L1, L2, rl2, part, parts)
-               : neigh_rows<false>(d, qa, stg, a0, ni, incl, start, excl, total, L0, L1, L2, rl2, part, parts);
+  if (frame) {
+    return neigh_rows_frame(d, qa, o, reinterpret_cast<float*>(stg), a0, ni, start, cnt, excl, total, L0, L1, L2, rl2, part, parts);
+  }
+  return neigh_rows_wrap(d, qa, stg, a0, ni, incl, start, excl, total, L0, L1, L2, rl2, part, parts);
 }
 
 __device__ __forceinline__ void neigh_cell_warp(const Dev& d, const uint4* qa, float4* stg, int c, float rl2) {
@@ -1945,7 +2079,7 @@ __global__ void k_copyback(Dev d) {
 constexpr int kNeighThreads = 128;
 __global__ void __launch_bounds__(kNeighThreads) k_neigh(Dev d, float rl2) {
   if (!d.g->any_rebuild || d.g->status) return;
-  __shared__ float4 stg[kNeighThreads / 32][kNStage];
+  __shared__ float4 stg[kNeighThreads / 32][kNSlice];
   const int w = (int)((blockIdx.x * (unsigned)blockDim.x + threadIdx.x) >> 5);
   if (w < d.ncell) neigh_cell_warp(d, d.q, stg[threadIdx.x >> 5], w, rl2);
 }

@@ -245,8 +245,8 @@ __global__ void __launch_bounds__(kPersThreads, kPersBlocksPerSm) k_persistent(c
       for (int i = tid; i < d.N; i += nth) copyback_item(d, i);
       phase_mark(d, s, 12);
       {  // the warp's candidate staging slice aliases the leg table (idle until the force phase)
-        static_assert(sizeof(LegTable) >= (kPersThreads / 32) * kNStage * sizeof(float4), "staging slices");
-        float4* stg = reinterpret_cast<float4*>(&T) + (threadIdx.x >> 5) * kNStage;
+        static_assert(sizeof(LegTable) >= (kPersThreads / 32) * kNSlice * sizeof(float4), "staging slices");
+        float4* stg = reinterpret_cast<float4*>(&T) + (threadIdx.x >> 5) * kNSlice;
         for (int c = gw; c < d.ncell; c += nwarps) neigh_cell_warp(d, d.tq, stg, c, P.rl2);
       }
       phase_mark(d, s, 13);
