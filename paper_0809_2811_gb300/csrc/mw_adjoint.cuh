@@ -187,7 +187,8 @@ __device__ void adjoint_block(const Dev& d, const AdjDev& A, const FParams& P, A
     L1 = bx.Lq[1];
     L2 = bx.Lq[2];
   }
-  const int nl = stage_legs<kG, kLMax>(d, P.rc2, T.ue, at, qi, L0, L1, L2, d.nbr + (size_t)(valid ? i : 0) * d.W, cnt);
+  const int nl = stage_legs<kG, kLMax>(d, P.rc2, T.ue, at, T.aux + (threadIdx.x >> 5) * kWAtoms * kLMax, qi, L0, L1, L2,
+                                         d.nbr + (size_t)(valid ? i : 0) * d.W, cnt);
   __syncwarp();
   const int nstage = nl <= kLMax ? nl : 0;  // larger centres: adjoint_overflow_item does everything
   // moments S0, s, M (xx yy zz xy xz yz) and their tangents

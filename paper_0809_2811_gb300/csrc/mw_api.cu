@@ -1534,7 +1534,7 @@ mw_status mw_step(mw_system* s, const mw_integrator* integ, int nsteps, mw_therm
     s->engine_used = eng;
     CluConfig clu;
     st = eng == MW_ENGINE_PERSISTENT
-             ? (cluster_config(s, &clu) ? run_cluster_engine(s, clu, nsteps, last, &fetched)
+             ? (cluster_config(s, nsteps, &clu) ? run_cluster_engine(s, clu, nsteps, last, &fetched)
                                         : run_persistent_engine(s, nsteps, last, &fetched))
              : run_graph_engine(s, nsteps, last, &fetched, eng == MW_ENGINE_PLAIN);
     s->g_known_valid = false;

@@ -284,7 +284,9 @@ __global__ void __launch_bounds__(kCluThreads, 2) k_cluster(const __grid_constan
     float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     for (int g = wid; g < gper; g += nwarp) {
       const int ic = off + ((int)rank * gper + g) * kWAtoms + lane / kG;
-      force_group<false, 0, kG, 0>(d, P, ue, aux, ic, ic < off + n && (int)rank * gper + g < ngrp, par, acc);
+      bool over = false;
+      force_group<false, 0, kG, 0>(d, P, ue, aux, ic, ic < off + n && (int)rank * gper + g < ngrp, acc, over);
+      if (over) force_overflow_item<false>(d, P, ic, par);
       __syncwarp();
     }
     clu_sync();

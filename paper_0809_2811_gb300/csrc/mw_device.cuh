@@ -1317,7 +1317,8 @@ constexpr int kG = 4;                    // lanes per centre in the leg phase
 constexpr int kFThreads = 128;
 constexpr int kFAtoms = kFThreads / kG;  // centres per block
 constexpr int kWAtoms = 32 / kG;         // centres per warp
-constexpr int kPre = 6;                  // neighbour slots per lane fetched ahead in the leg phase (8 spills at 64 registers)
+constexpr int kPre = 4;                  // neighbour slots per lane fetched ahead in the leg phase (k_force at 2^20 atoms:
+                                         // 206 us, 208 with 6, 219 with 8)
 
 // The force kernel's shared-memory leg table: a row of kRow float4 records
 // per centre (kRow a multiple of 8, i.e. of the 8 bank groups a quarter warp's
@@ -1328,8 +1329,11 @@ constexpr int kPre = 6;                  // neighbour slots per lane fetched ahe
 template <int kRow, int kCent = kFAtoms>
 struct LegTableT {
   static_assert(kRow % 8 == 0, "rows must cover whole sets of bank groups");
-  float4 ue[kCent * kRow];   // phase A: dx, dy, dz, j (int bits); then ux, uy, uz, ee
-  float4 aux[kCent * kRow];  // -1/2 dphi, nde, r, j (int bits)
+  // one species: dx, dy, dz, j (int bits); several: after phase B ux, uy, uz, ee
+  float4 ue[kCent * kRow];
+  // phase A: the rows' pieces; then, one species: ee, -1/2 dphi, nde, 1/r;
+  // several: -1/2 dphi, nde, r, j
+  float4 aux[kCent * kRow];
 };
 using LegTable = LegTableT<kLMax>;
 // Several species: a solute's larger cutoff gives its centres more legs, so
@@ -1434,63 +1438,83 @@ __device__ __noinline__ void force_overflow_item(const Dev& d, const FParams& P,
 
 // Leg phase A of one species (k_force and the adjoint): the KG lanes of a
 // centre walk its neighbour row and compact the pairs with r^2 < rc2 into the
-// centre's leg records tab(l) = (d, j), at most kLM of them; returns how many
-// there are.  Row entries and candidate positions are fetched for kPre slots
-// per lane before any is used (two memory latencies per batch instead of a
-// dependent chain per slot); every slot's test comes first, then one
-// compaction per batch (the lane's hits go to the group's running count plus
-// the hits of the group's lower lanes in this batch, in slot order).  Rows
-// longer than KG * kPre cost one more round trip per batch, not per slot.
-// Every lane of the warp calls it.
+// centre's leg records tab[at(l)] = (d, j), at most kLM of them; returns how
+// many there are.  The row is copied to shared memory first (kRowBuf entries
+// at a time, 16 bytes a lane, into warp_aux: the warp's own second records,
+// which no other warp may touch), then candidate positions are fetched
+// for kPre slots per lane before any is used; every slot's test comes first,
+// then one compaction per batch (the lane's hits go to the group's running
+// count plus the hits of the group's lower lanes in this batch, in slot
+// order).  Every lane of the warp calls it.
+// k_force is bound by the L1 data pipe (80 % busy): a row entry loaded by its
+// own lane, 4 bytes from each of 8 rows per warp, takes 8 times the pipe
+// slots of a 16-byte copy and a conflict-free shared-memory read.
+constexpr int kRowBuf = 92;  // ints a centre (of the 96 that kLMax records hold): 28 mod 32, so the 8 centres of a
+                             // warp (KG = 4) read their rows from disjoint banks, in whole 16-byte pieces
+__device__ __forceinline__ void cp_async16(int* dst, const int* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 template <int KG, int kLM, class At>
-__device__ __forceinline__ int stage_legs(const Dev& d, float rc2, float4* tab, At at, const uint4& qi, float L0, float L1,
-                                          float L2, const int* row, int cnt) {
+__device__ __forceinline__ int stage_legs(const Dev& d, float rc2, float4* tab, At at, float4* warp_aux, const uint4& qi,
+                                          float L0, float L1, float L2, const int* row, int cnt) {
+  static_assert(kRowBuf * 4 <= kLM * 16 && kRowBuf % 4 == 0, "the warp's row pieces fit its second records");
   const int lane = threadIdx.x & 31;
+  int* const rowbuf = reinterpret_cast<int*>(warp_aux) + (lane / KG) * kRowBuf;  // this centre's piece
   const int g = threadIdx.x & (KG - 1);
-  const int iters = __reduce_max_sync(kFull, (cnt + KG - 1) / KG);
+  const int longest = __reduce_max_sync(kFull, cnt);
   int nl = 0;
-  for (int t0 = 0; t0 < iters; t0 += kPre) {  // warp-uniform
-    int jr[kPre];
-    uint32_t qx[kPre], qy[kPre], qz[kPre];
-#pragma unroll
-    for (int t = 0; t < kPre; ++t) {
-      const int s = g + KG * (t0 + t);
-      jr[t] = (s < cnt) ? row[s] : -1;
+  for (int r0 = 0; r0 < longest; r0 += kRowBuf) {  // pieces of the rows (warp-uniform; one but for very long rows)
+    const int n = min(cnt - r0, kRowBuf);  // entries of this centre's piece (may be none)
+    if (r0 > 0) __syncwarp();  // the last piece's readers are done
+    if ((d.W & 3) == 0) {  // rows start on 16-byte boundaries (the last copy may read past cnt, inside the row)
+      for (int t = 4 * g; t < n; t += 4 * KG) cp_async16(rowbuf + t, row + r0 + t);
+      cp_async_wait();
+    } else {
+      for (int t = g; t < n; t += KG) rowbuf[t] = row[r0 + t];
     }
+    __syncwarp();
+    const int iters = (min(longest - r0, kRowBuf) + KG - 1) / KG;
+    for (int t0 = 0; t0 < iters; t0 += kPre) {  // warp-uniform
+      uint32_t qx[kPre], qy[kPre], qz[kPre];
 #pragma unroll
-    for (int t = 0; t < kPre; ++t) {
-      uint4 qj = make_uint4(0u, 0u, 0u, 0u);
-      if (jr[t] >= 0) qj = d.q[jr[t]];
-      qx[t] = qj.x;
-      qy[t] = qj.y;
-      qz[t] = qj.z;
-    }
-    float dx[kPre], dy[kPre], dz[kPre];
-    unsigned hits = 0u;  // bit t: slot t is a leg
-    int hc = 0;
-#pragma unroll
-    for (int t = 0; t < kPre; ++t) {
-      dx[t] = fix_diff(qi.x, qx[t], L0);
-      dy[t] = fix_diff(qi.y, qy[t], L1);
-      dz[t] = fix_diff(qi.z, qz[t], L2);
-      const bool hit = jr[t] >= 0 && fmaf(dx[t], dx[t], fmaf(dy[t], dy[t], dz[t] * dz[t])) < rc2;
-      hits |= hit ? 1u << t : 0u;
-      hc += hit ? 1 : 0;
-    }
-    int incl = hc;  // inclusive prefix of the hit counts over the group's lanes
-#pragma unroll
-    for (int o = 1; o < KG; o <<= 1) {
-      const int y = __shfl_up_sync(kFull, incl, o, KG);
-      if (g >= o) incl += y;
-    }
-    int pos = nl + incl - hc;
-#pragma unroll
-    for (int t = 0; t < kPre; ++t)
-      if ((hits >> t) & 1u) {
-        if (pos < kLM) tab[at(pos)] = make_float4(dx[t], dy[t], dz[t], __int_as_float(jr[t]));
-        ++pos;
+      for (int t = 0; t < kPre; ++t) {
+        const int s = g + KG * (t0 + t);
+        uint4 qj = make_uint4(0u, 0u, 0u, 0u);
+        if (s < n) qj = d.q[rowbuf[s]];
+        qx[t] = qj.x;
+        qy[t] = qj.y;
+        qz[t] = qj.z;
       }
-    nl += __shfl_sync(kFull, incl, lane | (KG - 1));  // the group's hits in this batch
+      float dx[kPre], dy[kPre], dz[kPre];
+      unsigned hits = 0u;  // bit t: slot t is a leg
+      int hc = 0;
+#pragma unroll
+      for (int t = 0; t < kPre; ++t) {
+        const int s = g + KG * (t0 + t);
+        dx[t] = fix_diff(qi.x, qx[t], L0);
+        dy[t] = fix_diff(qi.y, qy[t], L1);
+        dz[t] = fix_diff(qi.z, qz[t], L2);
+        const bool hit = s < n && fmaf(dx[t], dx[t], fmaf(dy[t], dy[t], dz[t] * dz[t])) < rc2;
+        hits |= hit ? 1u << t : 0u;
+        hc += hit ? 1 : 0;
+      }
+      int incl = hc;  // inclusive prefix of the hit counts over the group's lanes
+#pragma unroll
+      for (int o = 1; o < KG; o <<= 1) {
+        const int y = __shfl_up_sync(kFull, incl, o, KG);
+        if (g >= o) incl += y;
+      }
+      int pos = nl + incl - hc;
+#pragma unroll
+      for (int t = 0; t < kPre; ++t)
+        if ((hits >> t) & 1u) {
+          if (pos < kLM) tab[at(pos)] = make_float4(dx[t], dy[t], dz[t], __int_as_float(rowbuf[g + KG * (t0 + t)]));
+          ++pos;
+        }
+      nl += __shfl_sync(kFull, incl, lane | (KG - 1));  // the group's hits in this batch
+    }
   }
   return nl;
 }
@@ -1522,10 +1546,13 @@ __device__ __noinline__ int species_item(const Dev& d, const SpPair* sp, const f
 // force_group: the 32 / KG centres of one warp (centre i of this lane's
 // group; valid: there is one), ue and aux the warp's rows of the leg table;
 // adds to acc (E2, E3, W xx yy zz xy xz yz) and returns the centre's box.
-// Synchronises the warp only.
+// over: this lane leads a centre with more legs than the table holds, which
+// has added nothing; the caller hands it to force_overflow_item when its own
+// sums are done with (a call with them live would spill them).  Synchronises
+// the warp only.
 template <bool kCount, int kSp, int KG, int kOwn>
-__device__ __forceinline__ int force_group(const Dev& d, const FParams& P, float4* ue, float4* aux, int i, bool valid, int par,
-                                           float (&acc)[8], const SpPair* sps = nullptr, int nsp = 1,
+__device__ __forceinline__ int force_group(const Dev& d, const FParams& P, float4* ue, float4* aux, int i, bool valid,
+                                           float (&acc)[8], bool& over, const SpPair* sps = nullptr, int nsp = 1,
                                            const float2* stt = nullptr) {
   constexpr int kLM = kSp ? kLMaxSp : kLMax;  // legs staged per centre
   const int lane = threadIdx.x & 31;
@@ -1567,7 +1594,7 @@ __device__ __forceinline__ int force_group(const Dev& d, const FParams& P, float
       ue[at(l)] = make_float4(dx, dy, dz, __int_as_float(j));
     }
   } else if constexpr (kSp == 0) {
-    nl = stage_legs<KG, kLM>(d, P.rc2, ue, at, qi, L0, L1, L2, row, cnt);
+    nl = stage_legs<KG, kLM>(d, P.rc2, ue, at, aux, qi, L0, L1, L2, row, cnt);
   } else {
     const int iters = __reduce_max_sync(kFull, (cnt + KG - 1) / KG);
     const unsigned gsh = lane & ~(KG - 1);
@@ -1643,7 +1670,7 @@ __device__ __forceinline__ int force_group(const Dev& d, const FParams& P, float
       in = leg_terms(r2, P, lt);
     }
     if (!in) {  // FP32 rounding put it on the cutoff (or past its pair's): contributes nothing
-      *ue_p = make_float4(0.f, 0.f, 0.f, 0.f);
+      (kSp ? *ue_p : *ax_p) = make_float4(0.f, 0.f, 0.f, 0.f);
       continue;
     }
     if constexpr (kSp && kCount) ++nvalid;
@@ -1679,12 +1706,15 @@ __device__ __forceinline__ int force_group(const Dev& d, const FParams& P, float
         continue;
       }
     }
-    *ue_p = make_float4(ux, uy, uz, ee);
-    // (-1/2 dphi: the pair term's share of the virial, taken in phase C), nde, r, j
-    // (kSp = 2: j with the partner's species in bits 28-30)
-    const float jw = kSp == 2 ? __int_as_float(__float_as_int(ax_p->w) | (__float_as_int(ax_p->x) << 28))
-                              : (kSp ? ax_p->w : rec.w);
-    *ax_p = make_float4(-0.5f * dphi, lt.nde, r, jw);
+    // -1/2 dphi is the pair term's share of the virial, taken in phase C
+    if constexpr (kSp == 0) {
+      *ax_p = make_float4(ee, -0.5f * dphi, lt.nde, lt.invr);  // (the first record stays d and j)
+    } else {
+      *ue_p = make_float4(ux, uy, uz, ee);
+      // (kSp = 2: j with the partner's species in bits 28-30)
+      const float jw = kSp == 2 ? __int_as_float(__float_as_int(ax_p->w) | (__float_as_int(ax_p->x) << 28)) : ax_p->w;
+      *ax_p = make_float4(-0.5f * dphi, lt.nde, r, jw);
+    }
     if constexpr (kSp == 2) continue;  // no moments
     const float ex = ee * ux, ey = ee * uy, ez = ee * uz;
     m0 += ee;
@@ -1764,11 +1794,11 @@ __device__ __forceinline__ int force_group(const Dev& d, const FParams& P, float
   // a centre with one leg has no three-body term: its moments hold only that
   // leg, whose self term cancels up to rounding; the residue is not computed
   const bool three = nstage > 1;  // (uniform over the centre's lane group)
-  // the three-body force on the partner of leg (u, ee, nde, r) of a centre
+  // the three-body force on the partner of leg (u, ee, nde, tr = 2/r) of a centre
   // with moments (S0, s, M), and the leg's C; the k = j term is taken back
   // out with c_jj = |u|^2 as computed (not 1), so that it cancels the same
   // product inside the moments
-  auto leg_force = [&](float ux, float uy, float uz, float ee, float nde, float r, float S0, float sx, float sy,
+  auto leg_force = [&](float ux, float uy, float uz, float ee, float nde, float tr, float S0, float sx, float sy,
                        float sz, float Mxx, float Myy, float Mzz, float Mxy, float Mxz, float Myz, float& gx,
                        float& gy, float& gz) {
     const float mx = fmaf(Mxx, ux, fmaf(Mxy, uy, Mxz * uz));  // M u
@@ -1784,7 +1814,6 @@ __device__ __forceinline__ int force_group(const Dev& d, const FParams& P, float
     const float Ax = fmaf(-c0, sx, mx) - self * ux;
     const float Ay = fmaf(-c0, sy, my) - self * uy;
     const float Az = fmaf(-c0, sz, mz) - self * uz;
-    const float tr = 2.0f * rcp_approx(r);
     const float et = ee * tr;                       // ee_j tr_j
     const float cu = ee * fmaf(nde, Cj, tr * Bj);   // ee_j (nde_j C_j + tr_j B_j)
     gx = fmaf(cu, ux, -et * Ax);
@@ -1793,15 +1822,18 @@ __device__ __forceinline__ int force_group(const Dev& d, const FParams& P, float
     return Cj;
   };
   for (int l = g; l < nstage; l += KG) {
-    const float4 uj = ue[at(l)];
+    const float4 rec = ue[at(l)];
     const float4 xj = aux[at(l)];
-    const float ee = uj.w;
+    // the leg: its unit vector u, ee, -1/2 dphi, nde, 2 / r, its vector and partner
+    const float ee = kSp ? rec.w : xj.x;
     if (ee == 0.f) continue;  // leg dropped in phase B
-    const float r = xj.z;
-    const int j = __float_as_int(xj.w);
+    const float hd = kSp ? xj.x : xj.y, nde = kSp ? xj.y : xj.z;
+    const float tr = 2.0f * (kSp ? rcp_approx(xj.z) : xj.w);
+    const float3 uj = kSp ? make_float3(rec.x, rec.y, rec.z) : make_float3(rec.x * xj.w, rec.y * xj.w, rec.z * xj.w);
+    const int j = __float_as_int(kSp ? xj.w : rec.w);
     float gx = 0.f, gy = 0.f, gz = 0.f;
     if (three) {
-      const float Cj = leg_force(uj.x, uj.y, uj.z, ee, xj.y, r, m0, msx, msy, msz, mxx, myy, mzz, mxy, mxz, myz,
+      const float Cj = leg_force(uj.x, uj.y, uj.z, ee, nde, tr, m0, msx, msy, msz, mxx, myy, mzz, mxy, mxz, myz,
                                  gx, gy, gz);
       // the partner's share: scattered (pass 2: gathered by the partner, unless
       // it is a centre over the staged-leg limit)
@@ -1816,7 +1848,7 @@ __device__ __forceinline__ int force_group(const Dev& d, const FParams& P, float
         const float4 ma = d.mom[3 * (size_t)j], mb = d.mom[3 * (size_t)j + 1], mc = d.mom[3 * (size_t)j + 2];
         float hx, hy, hz;
         if (d.nleg[j] > 1) {
-          leg_force(-uj.x, -uj.y, -uj.z, ee, xj.y, r, ma.x, ma.y, ma.z, ma.w, mb.x, mb.y, mb.z, mb.w, mc.x, mc.y, hx,
+          leg_force(-uj.x, -uj.y, -uj.z, ee, nde, tr, ma.x, ma.y, ma.z, ma.w, mb.x, mb.y, mb.z, mb.w, mc.x, mc.y, hx,
                     hy, hz);
           fx += hx;
           fy += hy;
@@ -1825,9 +1857,9 @@ __device__ __forceinline__ int force_group(const Dev& d, const FParams& P, float
       }
     }
     // virial: r u_a (g_b - 1/2 dphi u_b), the three-body and the pair part
-    // (pass 2: xj.x = 0, the pair part was taken in pass 1)
-    const float hx = fmaf(xj.x, uj.x, gx), hy = fmaf(xj.x, uj.y, gy), hz = fmaf(xj.x, uj.z, gz);
-    const float rx = r * uj.x, ry = r * uj.y, rz = r * uj.z;
+    // (pass 2: hd = 0, the pair part was taken in pass 1)
+    const float hx = fmaf(hd, uj.x, gx), hy = fmaf(hd, uj.y, gy), hz = fmaf(hd, uj.z, gz);
+    const float rx = kSp ? xj.z * uj.x : rec.x, ry = kSp ? xj.z * uj.y : rec.y, rz = kSp ? xj.z * uj.z : rec.z;
     acc[2] = fmaf(rx, hx, acc[2]);
     acc[3] = fmaf(ry, hy, acc[3]);
     acc[4] = fmaf(rz, hz, acc[4]);
@@ -1845,13 +1877,10 @@ __device__ __forceinline__ int force_group(const Dev& d, const FParams& P, float
   }
   if (valid && g == 0) {
     red_add_v4(d.f + i, fx, fy, fz);
-    if (nl > kLM) {  // rare: more legs than the table holds
-      if constexpr (kSp != 0)
-        species_item<kCount>(d, sps, d.sp_tri, nsp, i, acc);
-      else
-        force_overflow_item<kCount>(d, P, i, par);
-    }
+    if constexpr (kSp != 0)
+      if (nl > kLM) species_item<kCount>(d, sps, d.sp_tri, nsp, i, acc);  // rare: more legs than the table holds
   }
+  if constexpr (kSp == 0) over = valid && g == 0 && nl > kLM;
   if (kCount && kOwn != 2) {  // legs and table-path triplets, one atomic per warp (pass 2 counts nothing)
     int nleg = nl;
     if constexpr (kSp) {  // legs inside their own pair's cutoff, summed over the group
@@ -1881,10 +1910,13 @@ __device__ void force_block(const Dev& d, const FParams& P,
                             const SpPair* sps = nullptr, int nsp = 1, const float2* stt = nullptr) {
   constexpr int kRows = (32 / KG) * (kSp ? kLMaxSp : kLMax);  // records of a warp's centres
   float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  bool over = false;
   const int w = (int)(threadIdx.x >> 5);
   const int i = blk * (kFThreads / KG) + (int)threadIdx.x / KG;
-  const int b = force_group<kCount, kSp, KG, kOwn>(d, P, T.ue + w * kRows, T.aux + w * kRows, i, i < d.N, par, acc, sps, nsp, stt);
+  const int b = force_group<kCount, kSp, KG, kOwn>(d, P, T.ue + w * kRows, T.aux + w * kRows, i, i < d.N, acc, over, sps, nsp, stt);
   box_accumulate<8>(acc, b, [&](int bb) { return &d.bst[bb].ew[par][0]; });
+  if constexpr (kSp == 0)
+    if (over) force_overflow_item<kCount>(d, P, i, par);  // rare
 }
 
 // k_force in several launch shapes, picked by the autotuner: KG lanes per
