@@ -460,7 +460,7 @@ void launch_rebuild(mw_system* s) {
   launch_scan(s);
   k_scatter<<<gb, kThreads, 0, s->stream>>>(d);
   k_copyback<<<std::max(gb, div_up(s->nbox, kThreads)), kThreads, 0, s->stream>>>(d);
-  k_neigh<<<div_up((long long)s->ncell * 32, kNeighThreads), kNeighThreads, 0, s->stream>>>(d, s->fp.rl2);
+  k_neigh<<<div_up((long long)s->ncell * 32, kNeighThreads), kNeighThreads, 0, s->stream>>>(d, s->fp.rl2, false);
 }
 
 void launch_force(mw_system* s) {
@@ -1916,8 +1916,8 @@ extern "C" mw_status mw_energy_forces_noalloc(int n, const double box[3], const 
   k_scan<<<1, kScanThreads, 0, sm>>>(d);
   k_na_scatter<<<gb, kThreads, 0, sm>>>(d, tq);
   Dev ds = d;  // the sorted view: neighbour list and forces work on the cell-sorted copy
-  ds.q = tq;
-  k_neigh<<<div_up(ncell * 32, kNeighThreads), kNeighThreads, 0, sm>>>(ds, tmp.fp.rl2);
+  ds.q = ds.tq = tq;
+  k_neigh<<<div_up(ncell * 32, kNeighThreads), kNeighThreads, 0, sm>>>(ds, tmp.fp.rl2, true);
   k_prep_force<<<gb, kThreads, 0, sm>>>(ds, 1);
   k_force<false><<<div_up(n, kFAtoms), kFThreads, 0, sm>>>(ds, tmp.fp);
   k_na_out<<<gb, kThreads, 0, sm>>>(ds, f_dev, energy_dev, virial_dev);

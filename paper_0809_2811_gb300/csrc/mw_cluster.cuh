@@ -120,9 +120,13 @@ __device__ __forceinline__ bool clu_rebuild(const Dev& d, CluShared& S, float4* 
   const Box& bx = S.bx;
   constexpr int T = kCluThreads;
   const int tid = (int)threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const bool sort = sorts(S.bs);  // (as scatter_item and copyback_item)
+  unsigned box = 0u;
   int c = 0, r = 0;
   if (on) {
-    c = cell_of(d.q[i], bx);
+    const uint4 q = d.q[i];
+    box = q.w;
+    c = cell_of(q, bx);
     r = atomicAdd(d.cell_cnt + c, 1);
   }
   clu_sync();
@@ -157,24 +161,32 @@ __device__ __forceinline__ bool clu_rebuild(const Dev& d, CluShared& S, float4* 
   else clu_sync();
   if (on) {
     const int p = (fits ? start[c - bx.cell_off] : __ldcg(d.cell_start + c)) + r;
+    uint4 q = d.q[i];
     if (p < bx.off || p >= bx.off + bx.n) {  // counts not cleared after an interrupted build: report, write nothing
       set_status(d.g, ST_CELLS);
       d.g->err_index = i;
     } else {
-      d.tx[p] = d.x[i]; d.ty[p] = d.y[i]; d.tz[p] = d.z[i];
-      d.tvx[p] = d.vx[i]; d.tvy[p] = d.vy[i]; d.tvz[p] = d.vz[i];
-      d.tid[p] = d.id[i];
-      d.tq[p] = d.q[i];
-      d.timg[p] = d.img[i];
+      if (sort) {
+        d.tx[p] = d.x[i]; d.ty[p] = d.y[i]; d.tz[p] = d.z[i];
+        d.tvx[p] = d.vx[i]; d.tvy[p] = d.vy[i]; d.tvz[p] = d.vz[i];
+        d.tid[p] = d.id[i];
+        d.timg[p] = d.img[i];
+        q.w = (unsigned)p;
+      } else {
+        d.qb[i] = q;
+        q.w = (unsigned)i;
+      }
+      d.tq[p] = q;
     }
   }
   clu_sync();
-  if (on) {
+  if (on && sort) {
     d.x[i] = d.tx[i]; d.y[i] = d.ty[i]; d.z[i] = d.tz[i];
     d.vx[i] = d.tvx[i]; d.vy[i] = d.tvy[i]; d.vz[i] = d.tvz[i];
     d.id[i] = d.tid[i];
     d.img[i] = d.timg[i];
-    const uint4 q = d.tq[i];
+    uint4 q = d.tq[i];
+    q.w = box;
     d.q[i] = q;
     d.qb[i] = q;
   }
@@ -185,7 +197,7 @@ __device__ __forceinline__ bool clu_rebuild(const Dev& d, CluShared& S, float4* 
   const int nw = (T >> 5) * (int)size;
   const int parts = max(1, min(4, nw / ncb));
   for (int k = wid * (int)size + (int)rank; k < ncb * parts; k += nw)
-    over |= neigh_cell(d, bx, d.tq, stg, bx.cell_off + k / parts, rl2, k % parts, parts);
+    over |= neigh_cell(d, bx, stg, bx.cell_off + k / parts, rl2, k % parts, parts);
   return over;
 }
 
@@ -275,6 +287,7 @@ __global__ void __launch_bounds__(kCluThreads, 2) k_cluster(const __grid_constan
       }
       if (tid == 0) {
         S.bs.rebuild = 0;
+        S.bs.sorted = 1;
         S.bs.rebuilds += 1;
         S.bs.Lb = S.bx.L[0];
         if (rank == 0) atomicOr(A.rebuild_bits + ((s - A.base) >> 5), 1u << ((s - A.base) & 31));

@@ -74,7 +74,7 @@ struct BoxState {   // mutated by kernels
   double ke_last;         // KE after the last end half, or of the state just set (kcal/mol)
   double s_endc;          // last end scale, still pending on the stored velocities
   float sig;              // S - 1 for the next kick1: S = s_endc times the start-half scale
-  int pad0_;
+  int sorted;             // 1: the box's atoms are in cell order of a recent build (see box_sorts)
   double ke_acc[2];       // per step-parity raw kinetic energy of v + a (the second half-kick)
   double ew[2][8];        // per step-parity E2, E3, W[6]
   int rebuild;            // displacement flag of this box
@@ -447,6 +447,26 @@ __device__ __forceinline__ void st_release(unsigned* p, unsigned v) {
 // flagged) are re-sorted and re-listed; the others keep their order and list
 // and never read their recomputed starts.
 __device__ __forceinline__ bool box_flagged(const Dev& d, int b) { return d.bst[b].rebuild != 0; }
+
+// Whether a build moves a box's atoms into cell order, or only builds the
+// list: every kSortEvery-th build, and the first after a new state or anything
+// else that flags every box.  The list is built from the cell-sorted copy tq,
+// whose records carry their atoms' indices, so it does not need the atoms
+// themselves in that order; they are sorted only so that a force block's
+// candidates lie close together, and in the 8 builds between (about 40 steps)
+// an atom diffuses well under a cell's width.  A build without the sort saves
+// moving each atom's 100 bytes twice: k_scatter + k_copyback 65 us at 2^20
+// atoms, 17 without.
+constexpr int kSortEvery = 8;
+__device__ __forceinline__ bool sorts(const BoxState& st) { return !st.sorted || st.rebuilds % kSortEvery == 0; }
+__device__ __forceinline__ bool box_sorts(const Dev& d, int b) { return sorts(d.bst[b]); }
+// A build of box b done (its scatter and copy-back have read the above).
+__device__ __forceinline__ void box_built(const Dev& d, int b) {
+  BoxState& st = d.bst[b];
+  st.sorted = 1;
+  st.rebuilds += 1;
+  st.Lb = d.box[b].L[0];
+}
 
 // Per-box accumulation of NV values held as FP32 by each thread; the sums
 // across blocks are FP64.  Every thread of the block calls it (b < 0 for
@@ -1049,7 +1069,7 @@ __device__ __forceinline__ bool neigh_count(const Dev& d, int mycount) {
 // batch located by a binary search over the 27 cells; 3 centres at a time 290 us).
 __device__ __forceinline__ bool neigh_rows_frame(const Dev& d, const uint4* qa, const uint4& o, float* stg, int a0, int ni, int first, int cnt,
                                                  int excl, int total, float L0, float L1, float L2, float rl2, int part,
-                                                 int parts) {
+                                                 int parts, bool slots) {
   static_assert(kNStage % 64 == 0, "whole groups of two candidates a lane");
   const int lane = threadIdx.x & 31;
   const unsigned below = (1u << lane) - 1u;  // lanes under this one
@@ -1066,7 +1086,9 @@ __device__ __forceinline__ bool neigh_rows_frame(const Dev& d, const uint4* qa, 
   }
   for (int ib = 0; ib < ni; ib += 32) {  // centre atoms of this cell, 32 at a time
     const int nb = min(32, ni - ib);
-    const uint4 qmine = qa[a0 + ib + min(lane, nb - 1)];  // lane k's centre
+    const int ms = a0 + ib + min(lane, nb - 1);
+    const uint4 qmine = qa[ms];  // lane k's centre
+    const int me = slots ? ms : (int)qmine.w;  // and its index
     const float cx = fix_diff(qmine.x, o.x, L0), cy = fix_diff(qmine.y, o.y, L1), cz = fix_diff(qmine.z, o.z, L2);  // o - centre
     int mycount = 0;  // neighbours of lane k's centre so far
     for (int c0 = 0; c0 < total; c0 += kNStage) {  // chunks of the candidate list (warp-uniform)
@@ -1089,6 +1111,7 @@ __device__ __forceinline__ bool neigh_rows_frame(const Dev& d, const uint4* qa, 
         if (t < nch) {
           j = c0 + t + delta[r];
           const uint4 qj = qa[j];
+          if (!slots) j = (int)qj.w;
           x = fix_diff(o.x, qj.x, L0);
           y = fix_diff(o.y, qj.y, L1);
           z = fix_diff(o.z, qj.z, L2);
@@ -1115,9 +1138,9 @@ __device__ __forceinline__ bool neigh_rows_frame(const Dev& d, const uint4* qa, 
           xc[c] = pk2(x, x);
           yc[c] = pk2(y, y);
           zc[c] = pk2(z, z);
-          ic[c] = a0 + ib + kc;
+          ic[c] = __shfl_sync(kFull, me, kc);
           cc[c] = __shfl_sync(kFull, mycount, kc);
-          rc[c] = d.nbr + (size_t)(a0 + ib + kc) * d.W;
+          rc[c] = d.nbr + (size_t)ic[c] * d.W;
         }
         for (int gr = 0; gr < ngrp; ++gr) {
           const int at = (gr << 6) + 2 * lane;
@@ -1153,7 +1176,7 @@ __device__ __forceinline__ bool neigh_rows_frame(const Dev& d, const uint4* qa, 
           if (on[c] && lane == k + c) mycount = cc[c];
       }
     }
-    if (lane < nb && (lane / kNeighCentres) % parts == part) d.nbr_cnt[a0 + ib + lane] = mycount;
+    if (lane < nb && (lane / kNeighCentres) % parts == part) d.nbr_cnt[me] = mycount;
     over |= neigh_count(d, mycount);
   }
   return over;
@@ -1165,13 +1188,15 @@ __device__ __forceinline__ bool neigh_rows_frame(const Dev& d, const uint4* qa, 
 // fixed-point; entries past the last candidate get j = -1.
 __device__ __forceinline__ bool neigh_rows_wrap(const Dev& d, const uint4* qa, float4* stg, int a0, int ni, int incl, int start,
                                                 int excl, int total, float L0, float L1, float L2, float rl2, int part,
-                                                int parts) {
+                                                int parts, bool slots) {
   const int lane = threadIdx.x & 31;
   const unsigned below = (1u << lane) - 1u;  // lanes under this one
   bool over = false;
   for (int ib = 0; ib < ni; ib += 32) {  // centre atoms of this cell, 32 at a time
     const int nb = min(32, ni - ib);
-    const uint4 qmine = qa[a0 + ib + min(lane, nb - 1)];  // lane k's centre
+    const int ms = a0 + ib + min(lane, nb - 1);
+    const uint4 qmine = qa[ms];  // lane k's centre
+    const int me = slots ? ms : (int)qmine.w;  // and its index
     int mycount = 0;  // neighbours of lane k's centre so far
     for (int c0 = 0; c0 < total; c0 += kNStage) {  // chunks of the candidate list (warp-uniform)
       const int nch = min(kNStage, total - c0);
@@ -1192,7 +1217,8 @@ __device__ __forceinline__ bool neigh_rows_wrap(const Dev& d, const uint4* qa, f
         if (t < total) {
           const int j = sk + (t - ek);
           const uint4 qj = qa[j];
-          e = make_float4(__uint_as_float(qj.x), __uint_as_float(qj.y), __uint_as_float(qj.z), __int_as_float(j));
+          e = make_float4(__uint_as_float(qj.x), __uint_as_float(qj.y), __uint_as_float(qj.z),
+                          slots ? __int_as_float(j) : __uint_as_float(qj.w));
         }
         stg[(bt << 5) + lane] = e;
       }
@@ -1201,7 +1227,7 @@ __device__ __forceinline__ bool neigh_rows_wrap(const Dev& d, const uint4* qa, f
         if ((k / kNeighCentres) % parts != part) continue;
         const uint32_t xc = __shfl_sync(kFull, qmine.x, k), yc = __shfl_sync(kFull, qmine.y, k), zc = __shfl_sync(kFull, qmine.z, k);
         int cc = __shfl_sync(kFull, mycount, k);
-        const int ic = a0 + ib + k;
+        const int ic = __shfl_sync(kFull, me, k);
         int* const rc = d.nbr + (size_t)ic * d.W;
         for (int bt = 0; bt < nbat; ++bt) {
           const float4 e = stg[(bt << 5) + lane];
@@ -1214,7 +1240,7 @@ __device__ __forceinline__ bool neigh_rows_wrap(const Dev& d, const uint4* qa, f
         if (lane == k) mycount = cc;
       }
     }
-    if (lane < nb && (lane / kNeighCentres) % parts == part) d.nbr_cnt[a0 + ib + lane] = mycount;
+    if (lane < nb && (lane / kNeighCentres) % parts == part) d.nbr_cnt[me] = mycount;
     over |= neigh_count(d, mycount);
   }
   return over;
@@ -1225,8 +1251,9 @@ __device__ __forceinline__ bool neigh_rows_wrap(const Dev& d, const uint4* qa, f
 // for itself and taking every parts-th group of kNeighCentres centres (a
 // build with fewer cells than warps is as long as one cell's chain of
 // dependent batches).  Returns whether a row was wider than its allocation.
-__device__ bool neigh_cell(const Dev& d, const Box& bx, const uint4* qa, float4* stg, int c, float rl2, int part = 0,
-                           int parts = 1) {
+__device__ bool neigh_cell(const Dev& d, const Box& bx, float4* stg, int c, float rl2, int part = 0, int parts = 1,
+                           bool slots = false) {
+  const uint4* const qa = d.tq;  // cell-sorted positions; w: the atom's index (slots: its place)
   const int lane = threadIdx.x & 31;
   const int a0 = d.cell_start[c];
   const int ni = d.cell_start[c + 1] - a0;
@@ -1275,14 +1302,14 @@ __device__ bool neigh_cell(const Dev& d, const Box& bx, const uint4* qa, float4*
   const int excl = incl - cnt;
   const int total = __shfl_sync(kFull, incl, 31);
   if (frame) {
-    return neigh_rows_frame(d, qa, o, reinterpret_cast<float*>(stg), a0, ni, start, cnt, excl, total, L0, L1, L2, rl2, part, parts);
+    return neigh_rows_frame(d, qa, o, reinterpret_cast<float*>(stg), a0, ni, start, cnt, excl, total, L0, L1, L2, rl2, part, parts, slots);
   }
-  return neigh_rows_wrap(d, qa, stg, a0, ni, incl, start, excl, total, L0, L1, L2, rl2, part, parts);
+  return neigh_rows_wrap(d, qa, stg, a0, ni, incl, start, excl, total, L0, L1, L2, rl2, part, parts, slots);
 }
 
-__device__ __forceinline__ void neigh_cell_warp(const Dev& d, const uint4* qa, float4* stg, int c, float rl2) {
+__device__ __forceinline__ void neigh_cell_warp(const Dev& d, float4* stg, int c, float rl2, bool slots = false) {
   const int b = d.cell_box[c];
-  if (box_flagged(d, b)) neigh_cell(d, d.box[b], qa, stg, c, rl2);  // warp-uniform
+  if (box_flagged(d, b)) neigh_cell(d, d.box[b], stg, c, rl2, 0, 1, slots);  // warp-uniform
 }
 
 // ---------------------------------------------------------------------------
@@ -1999,32 +2026,45 @@ __device__ __forceinline__ void bin_item(const Dev& d, int i) {
   d.rank[i] = atomicAdd(d.cell_cnt + c, 1);
 }
 
-// a2: atom i to its sorted slot in the staging arrays.
+// a2: atom i to its sorted slot in the staging arrays: its position with its
+// index (the list is built from these), and, when the box sorts its atoms,
+// the rest of its state.  Otherwise the build position is recorded here.
 __device__ __forceinline__ void scatter_item(const Dev& d, int i) {
-  if (!box_flagged(d, (int)d.q[i].w)) return;
+  uint4 q = d.q[i];
+  const int b = (int)q.w;
+  if (!box_flagged(d, b)) return;
   const int p = d.cell_start[d.cell[i]] + d.rank[i];
   if ((unsigned)p >= (unsigned)d.N) {  // counts not cleared after an interrupted build: report, write nothing
     set_status(d.g, ST_CELLS);
     d.g->err_index = i;
     return;
   }
-  d.tx[p] = d.x[i]; d.ty[p] = d.y[i]; d.tz[p] = d.z[i];
-  d.tvx[p] = d.vx[i]; d.tvy[p] = d.vy[i]; d.tvz[p] = d.vz[i];
-  d.tid[p] = d.id[i];
-  d.tq[p] = d.q[i];
-  d.timg[p] = d.img[i];
-  if (d.typ) d.ttyp[p] = d.typ[i];
+  if (box_sorts(d, b)) {
+    d.tx[p] = d.x[i]; d.ty[p] = d.y[i]; d.tz[p] = d.z[i];
+    d.tvx[p] = d.vx[i]; d.tvy[p] = d.vy[i]; d.tvz[p] = d.vz[i];
+    d.tid[p] = d.id[i];
+    d.timg[p] = d.img[i];
+    if (d.typ) d.ttyp[p] = d.typ[i];
+    q.w = (unsigned)p;
+  } else {
+    d.qb[i] = q;
+    q.w = (unsigned)i;
+  }
+  d.tq[p] = q;
 }
 
-// a2: staging arrays back to the state arrays; build positions recorded.
+// a2: staging arrays back to the state arrays of a box that sorts; build
+// positions recorded.
 __device__ __forceinline__ void copyback_item(const Dev& d, int i) {
-  if (!box_flagged(d, (int)d.q[i].w)) return;  // a box keeps its atom range
+  const int b = (int)d.q[i].w;  // a box keeps its atom range
+  if (!box_flagged(d, b) || !box_sorts(d, b)) return;
   d.x[i] = d.tx[i]; d.y[i] = d.ty[i]; d.z[i] = d.tz[i];
   d.vx[i] = d.tvx[i]; d.vy[i] = d.tvy[i]; d.vz[i] = d.tvz[i];
   d.id[i] = d.tid[i];
   d.img[i] = d.timg[i];
   if (d.typ) d.typ[i] = d.ttyp[i];
-  const uint4 q = d.tq[i];
+  uint4 q = d.tq[i];
+  q.w = (unsigned)b;
   d.q[i] = q;
   d.qb[i] = q;
 }
@@ -2101,19 +2141,19 @@ __global__ void k_copyback(Dev d) {
   if (!d.g->any_rebuild || d.g->status) return;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i == 0) d.g->rebuild_steps += 1;
-  if (i < d.nbox && box_flagged(d, i)) {
-    d.bst[i].rebuilds += 1;
-    d.bst[i].Lb = d.box[i].L[0];
-  }
   if (i < d.N) copyback_item(d, i);
 }
 
 constexpr int kNeighThreads = 128;
-__global__ void __launch_bounds__(kNeighThreads) k_neigh(Dev d, float rl2) {
+// slots: the records of d.tq carry no indices, an atom's place is its index
+// (the entry point that cannot allocate).
+__global__ void __launch_bounds__(kNeighThreads) k_neigh(Dev d, float rl2, bool slots) {
   if (!d.g->any_rebuild || d.g->status) return;
   __shared__ float4 stg[kNeighThreads / 32][kNSlice];
   const int w = (int)((blockIdx.x * (unsigned)blockDim.x + threadIdx.x) >> 5);
-  if (w < d.ncell) neigh_cell_warp(d, d.q, stg[threadIdx.x >> 5], w, rl2);
+  if (w < d.ncell) neigh_cell_warp(d, stg[threadIdx.x >> 5], w, rl2, slots);
+  const int b = (int)(blockIdx.x * blockDim.x + threadIdx.x);  // (there are at least as many threads as boxes)
+  if (b < d.nbox && box_flagged(d, b)) box_built(d, b);
 }
 
 
@@ -2471,7 +2511,10 @@ __global__ void k_flush_pending(Dev d) {
 // Flags every box for a rebuild (new state, parameters, skin or list width).
 __global__ void k_flag_all(Dev d) {
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b < d.nbox) d.bst[b].rebuild = 1;
+  if (b < d.nbox) {
+    d.bst[b].rebuild = 1;
+    d.bst[b].sorted = 0;
+  }
   if (b == 0) d.g->any_rebuild = 1;
 }
 

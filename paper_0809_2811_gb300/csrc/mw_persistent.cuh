@@ -228,7 +228,8 @@ __global__ void __launch_bounds__(kPersThreads, kPersBlocksPerSm) k_persistent(c
     }
     phase_mark(d, s, 2);
     // a2 + a3: cell binning and neighbour list, when due (flag is stable until kick2)
-    if (*(volatile int*)&g->any_rebuild) {
+    const bool listed = *(volatile int*)&g->any_rebuild != 0;
+    if (listed) {
       if (tid == 0) g->max_count = 0;
       for (int i = tid; i < d.N; i += nth) bin_item(d, i);
       phase_mark(d, s, 8);
@@ -247,13 +248,9 @@ __global__ void __launch_bounds__(kPersThreads, kPersBlocksPerSm) k_persistent(c
       {  // the warp's candidate staging slice aliases the leg table (idle until the force phase)
         static_assert(sizeof(LegTable) >= (kPersThreads / 32) * kNSlice * sizeof(float4), "staging slices");
         float4* stg = reinterpret_cast<float4*>(&T) + (threadIdx.x >> 5) * kNSlice;
-        for (int c = gw; c < d.ncell; c += nwarps) neigh_cell_warp(d, d.tq, stg, c, P.rl2);
+        for (int c = gw; c < d.ncell; c += nwarps) neigh_cell_warp(d, stg, c, P.rl2);
       }
       phase_mark(d, s, 13);
-      if (tid < d.nbox && box_flagged(d, tid)) {
-        d.bst[tid].rebuilds += 1;
-        d.bst[tid].Lb = d.box[tid].L[0];
-      }
       if (tid == 0) g->rebuild_steps += 1;
       if (grid_barrier(g, gen, wait_ns)) return;
     }
@@ -266,7 +263,10 @@ __global__ void __launch_bounds__(kPersThreads, kPersBlocksPerSm) k_persistent(c
     phase_mark(d, s, 5);
     // a7 second half: kinetic energy of v + a per box; the rebuild (if any) is consumed
     if (blockIdx.x == 0) {
-      for (int k = threadIdx.x; k < d.nbox; k += blockDim.x) d.bst[k].rebuild = 0;
+      for (int k = threadIdx.x; k < d.nbox; k += blockDim.x) {
+        if (listed && box_flagged(d, k)) box_built(d, k);
+        d.bst[k].rebuild = 0;
+      }
       if (threadIdx.x == 0) g->any_rebuild = 0;
     }
     for (int i0 = blockIdx.x * kPersThreads; i0 < d.N; i0 += nth) {  // block-uniform
