@@ -85,7 +85,7 @@ typedef enum mw_thermostat { MW_NVE = 0, MW_BERENDSEN = 1, MW_NOSE_HOOVER = 2, M
  * steps with grid-wide barriers between phases; mw_step runs small boxes, and
  * batches of them, in one thread-block cluster per box instead (the library
  * picks by size; same results to rounding).  AUTO: the library picks
- * (the autotuner's choice when one was made, else PERSISTENT).  PLAIN: the
+ * (the autotuner's choice when one was made, else by size).  PLAIN: the
  * plain GPU path the others are measured against: every phase kernel
  * launched from the host every step (no graph, no persistent launch) and a
  * force kernel with one thread per atom looping over its leg pairs (leg

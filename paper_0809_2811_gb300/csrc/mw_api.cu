@@ -1518,6 +1518,19 @@ mw_status mw_forces_async(mw_system* s) {
   return MW_OK;
 }
 
+// The engine of MW_ENGINE_AUTO where no autotuner has chosen: the persistent
+// one, above 150000 atoms the graph engine.  The grid-wide kernel runs every
+// phase at the force phase's 20 warps an SM; from about 10^5 atoms on the
+// separate kernels' 32 are worth more than the launches between them (20
+// steps, skin 1 A: 65536 atoms 1065 us persistent, 1194 graph; 100000 1424 /
+// 1419; 200000 2418 / 2356; 400000 4778 / 4447; 256 uneven boxes of 1.16 10^6
+// atoms 11808 / 10455).  Isobaric runs stay: the persistent tail is quicker
+// (64000 atoms 2024 / 2753).
+static int auto_engine(const mw_system* s) {
+  if (s->tuned_engine >= 0) return s->tuned_engine;
+  return s->N > 150000 && s->integ.kind != TH_NPT ? MW_ENGINE_GRAPH : MW_ENGINE_PERSISTENT;
+}
+
 mw_status mw_step(mw_system* s, const mw_integrator* integ, int nsteps, mw_thermo* last) {
   Range range_("mw_step");
   if (!s) return fail(MW_EINVAL, "system is NULL");
@@ -1529,7 +1542,7 @@ mw_status mw_step(mw_system* s, const mw_integrator* integ, int nsteps, mw_therm
   bool fetched = false;  // the run's last record came back with its final status read
   if (nsteps > 0) {
     int eng = s->engine;
-    if (eng == MW_ENGINE_AUTO) eng = s->tuned_engine >= 0 ? s->tuned_engine : MW_ENGINE_PERSISTENT;
+    if (eng == MW_ENGINE_AUTO) eng = auto_engine(s);
     if (eng == MW_ENGINE_PERSISTENT && !persistent_available(s)) eng = MW_ENGINE_GRAPH;
     s->engine_used = eng;
     CluConfig clu;
@@ -1558,7 +1571,7 @@ mw_status mw_step_async(mw_system* s, const mw_integrator* integ, int nsteps) {
   if ((st = ensure_forces(s)) != MW_OK) return st;
   if (nsteps == 0) return MW_OK;
   int eng = s->engine;
-  if (eng == MW_ENGINE_AUTO) eng = s->tuned_engine >= 0 ? s->tuned_engine : MW_ENGINE_PERSISTENT;
+  if (eng == MW_ENGINE_AUTO) eng = auto_engine(s);
   if (eng == MW_ENGINE_PERSISTENT && !persistent_available(s)) eng = MW_ENGINE_GRAPH;
   s->engine_used = eng;
   if ((st = prime_thermostat(s)) != MW_OK) return st;
