@@ -80,6 +80,10 @@ struct mw_system {
   // flags every box for a rebuild, by a failed run, by isobaric steps):
   // mw_set_state may then keep them (k_load_state_keep)
   bool order_ok = false;
+  // a state set in the kept order moved no atom past its list's margin (read
+  // back with the state's status): the next force call needs no build.
+  // Cleared by anything that flags a box.
+  bool lists_current = false;
   double* eout = nullptr;  // 9 * nbox doubles: energies + virials staging
   Dev d{};
   FParams fp{};
@@ -339,6 +343,7 @@ mw_status flush_pending(mw_system* s) {
 
 mw_status flag_all(mw_system* s) {
   s->order_ok = false;
+  s->lists_current = false;
   k_flag_all<<<div_up(s->nbox, kThreads), kThreads, 0, s->stream>>>(s->d);
   MW_CUDA(cudaGetLastError());
   return MW_OK;
@@ -443,11 +448,19 @@ void launch_kick2(mw_system* s) {
     k_kick2<false><<<kb, kKThreads, 0, s->stream>>>(s->d);
 }
 
+// Cells that one block scans in one launch (a pass of 8 cells a thread): up to
+// here about 4 us, two launches of the chunked scan 6 + 6 us at 5832 cells.
+constexpr int kScanOneBlock = 8 * kScanThreads;
+
 // Blocks of the two-kernel cell scan: about 512 cells each, at most the
 // chunk buffer's capacity.
 int scan_blocks(const mw_system* s) { return std::max(1, std::min(s->d.chunk_cap, div_up(s->ncell, 512))); }
 
 void launch_scan(mw_system* s) {
+  if (s->ncell <= kScanOneBlock) {
+    k_scan<<<1, kScanThreads, 0, s->stream>>>(s->d);
+    return;
+  }
   const int sb = scan_blocks(s);
   k_scan_local<<<sb, kPersThreads, 0, s->stream>>>(s->d);
   k_scan_offsets<<<sb, kPersThreads, 0, s->stream>>>(s->d);
@@ -596,24 +609,39 @@ mw_status grow_nbr_after_overflow(mw_system* s, const Global& g) {
   return alloc_nbr(s, w);
 }
 
-// Forces (and the thermo snapshot) at the current positions, with overflow recovery.
-mw_status ensure_forces(mw_system* s) {
+// Forces (and the thermo snapshot) at the current positions, with overflow
+// recovery.  out: what the caller wants of them, written in the same launch
+// sequence (complete on return; untouched after an error).  prepared: the
+// caller's kernel has done k_prep_force's work.
+mw_status ensure_forces(mw_system* s, const ForceOut* out = nullptr, bool prepared = false) {
   if (!s->state_set) return fail(MW_ESTATE, "no state set (call mw_set_state first)");
-  if (s->forces_valid) return MW_OK;
+  const ForceOut o = out ? *out : ForceOut{};
+  const int go = div_up((o.f64 || o.f32) ? std::max(s->N, s->nbox) : s->nbox, kThreads);
   mw_status st;
-  if ((st = flush_pending(s)) != MW_OK) return st;
-  if ((st = set_func_attrs()) != MW_OK) return st;
-  for (int attempt = 0; attempt < 4; ++attempt) {
-    k_prep_force<<<div_up(std::max(s->N, s->nbox), kThreads), kThreads, 0, s->stream>>>(s->d, 1);
+  if (s->forces_valid) {
+    if (!out) return MW_OK;
+    k_force_out<<<go, kThreads, 0, s->stream>>>(s->d, o, false);
     MW_CUDA(cudaGetLastError());
-    launch_rebuild(s);
+    MW_CUDA(cudaStreamSynchronize(s->stream));
+    return MW_OK;
+  }
+  if ((st = set_func_attrs()) != MW_OK) return st;
+  // a state just set in the kept order may have told that no list is stale
+  const bool rebuild = !s->lists_current;
+  s->lists_current = false;
+  for (int attempt = 0; attempt < 4; ++attempt) {
+    if (!prepared || attempt > 0)  // (with the pending half-kick)
+      k_prep_force<<<div_up(std::max(s->N, s->nbox), kThreads), kThreads, 0, s->stream>>>(s->d, attempt == 0 ? 2 : 1);
+    MW_CUDA(cudaGetLastError());
+    if (attempt == 0 && (st = set_global_field(s, offsetof(Global, pend), 0)) != MW_OK) return st;
+    if (rebuild || attempt > 0) launch_rebuild(s);
     launch_force(s);
     if (s->v_pending) {  // velocities of a state just set (their copy ran beside this force call)
       MW_CUDA(cudaStreamWaitEvent(s->stream, s->copy_ev[1], 0));
       k_load_velocities_keep<<<div_up(s->N, kThreads), kThreads, 0, s->stream>>>(s->d, s->d.stage2);
       s->v_pending = false;
     }
-    k_thermo_snapshot<<<div_up(s->nbox, kThreads), kThreads, 0, s->stream>>>(s->d);
+    k_force_out<<<go, kThreads, 0, s->stream>>>(s->d, o, true);
     MW_CUDA(cudaGetLastError());
     Global g;
     if ((st = read_global(s, &g)) != MW_OK) return st;
@@ -795,8 +823,6 @@ mw_status copy_lane(mw_system* s) {
   return MW_OK;
 }
 
-mw_status ensure_forces(mw_system* s);
-
 // mw_set_state in the kept order with host velocities: the positions are
 // copied and loaded, and the force call at them (which the next step or
 // energy call would make) runs while the velocities are copied in on the
@@ -851,6 +877,7 @@ mw_status do_set_state(mw_system* s, const double* x, const double* v, bool dev)
   const double* xd = x;
   const double* vd = v;
   const bool keep = s->state_set && s->order_ok && s->integ.kind != TH_NPT;
+  s->lists_current = false;
   if (!dev && keep && v) return set_state_keep_overlapped(s, x, v, bytes);
   if (!dev && keep) {
     // the current order is kept, so the loading kernel reads the inputs
@@ -914,6 +941,7 @@ mw_status do_set_state(mw_system* s, const double* x, const double* v, bool dev)
     return fail(MW_EINVAL, "non-finite position or velocity of atom %d", gh.err_index);
   }
   if (!keep) s->order_ok = false;  // identity order: sorted and listed by the next force call
+  s->lists_current = keep && !gh.any_rebuild;
   s->state_set = true;
   s->forces_valid = false;
   s->need_prime = true;  // thermostat at rest: xi = eta = 0, KE of the new velocities
@@ -1467,21 +1495,15 @@ mw_status mw_get_neighbors(mw_system* s, int* counts, int* nbr, int width) {
 mw_status mw_energy_forces(mw_system* s, double* f, double* energy, double* virial) {
   Range range_("mw_energy_forces");
   if (!s) return fail(MW_EINVAL, "system is NULL");
+  ForceOut o;
+  if (f) o.f64 = s->d.stage;
+  if (energy) o.e = s->eout;
+  if (virial) o.w = s->eout + 3 * (size_t)s->nbox;
   mw_status st;
-  if ((st = ensure_forces(s)) != MW_OK) return st;
-  if (f) {
-    k_gather_forces<<<div_up(s->N, kThreads), kThreads, 0, s->stream>>>(s->d, s->d.stage, nullptr);
-    MW_CUDA(cudaGetLastError());
-    MW_CUDA(cudaMemcpyAsync(f, s->d.stage, sizeof(double) * 3 * (size_t)s->N, cudaMemcpyDeviceToHost, s->stream));
-  }
-  if (energy || virial) {
-    double* e = s->eout;
-    double* w = s->eout + 3 * (size_t)s->nbox;
-    k_energy_out<<<div_up(s->nbox, kThreads), kThreads, 0, s->stream>>>(s->d, e, w);
-    MW_CUDA(cudaGetLastError());
-    if (energy) MW_CUDA(cudaMemcpyAsync(energy, e, sizeof(double) * 3 * s->nbox, cudaMemcpyDeviceToHost, s->stream));
-    if (virial) MW_CUDA(cudaMemcpyAsync(virial, w, sizeof(double) * 6 * s->nbox, cudaMemcpyDeviceToHost, s->stream));
-  }
+  if ((st = ensure_forces(s, &o)) != MW_OK) return st;
+  if (f) MW_CUDA(cudaMemcpyAsync(f, o.f64, sizeof(double) * 3 * (size_t)s->N, cudaMemcpyDeviceToHost, s->stream));
+  if (energy) MW_CUDA(cudaMemcpyAsync(energy, o.e, sizeof(double) * 3 * s->nbox, cudaMemcpyDeviceToHost, s->stream));
+  if (virial) MW_CUDA(cudaMemcpyAsync(virial, o.w, sizeof(double) * 6 * s->nbox, cudaMemcpyDeviceToHost, s->stream));
   MW_CUDA(cudaStreamSynchronize(s->stream));
   return MW_OK;
 }
@@ -1491,21 +1513,17 @@ mw_status mw_energy_forces_dev(mw_system* s, const double* x_dev, float* f_dev, 
   if (!s) return fail(MW_EINVAL, "system is NULL");
   if (x_dev) {
     if (!s->state_set) return do_set_state(s, x_dev, nullptr, true) == MW_OK ? mw_energy_forces_dev(s, nullptr, f_dev, energy_dev, virial_dev) : MW_ECUDA;
-    mw_status st;
-    if ((st = flush_pending(s)) != MW_OK) return st;
-    k_load_positions<<<div_up(s->N, kThreads), kThreads, 0, s->stream>>>(s->d, x_dev, s->boxid);
+    k_load_positions<<<div_up(std::max(s->N, s->nbox), kThreads), kThreads, 0, s->stream>>>(s->d, x_dev, s->boxid);
     MW_CUDA(cudaGetLastError());
-    if ((st = flag_all(s)) != MW_OK) return st;
+    s->order_ok = false;
+    s->lists_current = false;
     s->forces_valid = false;
   }
-  mw_status st;
-  if ((st = ensure_forces(s)) != MW_OK) return st;
-  if (f_dev) k_gather_forces<<<div_up(s->N, kThreads), kThreads, 0, s->stream>>>(s->d, nullptr, f_dev);
-  if (energy_dev || virial_dev)
-    k_energy_out<<<div_up(s->nbox, kThreads), kThreads, 0, s->stream>>>(s->d, energy_dev, virial_dev);
-  MW_CUDA(cudaGetLastError());
-  MW_CUDA(cudaStreamSynchronize(s->stream));
-  return MW_OK;
+  ForceOut o;
+  o.f32 = f_dev;
+  o.e = energy_dev;
+  o.w = virial_dev;
+  return ensure_forces(s, &o, x_dev != nullptr);
 }
 
 mw_status mw_forces_async(mw_system* s) {

@@ -2272,12 +2272,42 @@ __global__ void k_record_at(Dev d, int pp) {
 // ---------------------------------------------------------------------------
 // Setup / IO kernels.
 
+// Applies a pending second half-kick (v += dt/2 F/m) to atom i, before
+// anything changes the forces or the atom order outside a step.
+__device__ __forceinline__ void flush_atom(const Dev& d, double cf, int i) {
+  const float4 F = d.f[i];
+  d.vx[i] = split_df(join_df(d.vx[i]) + cf * F.x);
+  d.vy[i] = split_df(join_df(d.vy[i]) + cf * F.y);
+  d.vz[i] = split_df(join_df(d.vz[i]) + cf * F.z);
+}
+// Before a force call outside a step: the accumulators of this parity and the
+// counters start from zero.
+__device__ __forceinline__ void prep_box(const Dev& d, int i) {
+  const int par = (int)(d.g->step & 1ull);
+  if (i == 0) {
+    d.g->n_over = 0;
+    d.g->npairs = 0;
+    d.g->ntrip = 0;
+  }
+  if (i < d.nbox)
+    for (int k = 0; k < 8; ++k) d.bst[i].ew[par][k] = 0.0;
+}
 // New positions for the current atom order (mw_energy_forces_dev): from a
 // user-order AoS device array into the sorted arrays, x[i] = xin[id[i]],
-// wrapped into [0, L); q recomputed.
+// wrapped into [0, L); q recomputed.  Also flags every box for a rebuild and
+// does what k_prep_force does (one launch instead of four: a small box's
+// force call is as long as its launches).
 __global__ void k_load_positions(Dev d, const double* __restrict__ xin, const int* __restrict__ boxid) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  prep_box(d, i);
+  if (i < d.nbox) {  // every list is stale
+    d.bst[i].rebuild = 1;
+    d.bst[i].sorted = 0;
+  }
+  if (i == 0) d.g->any_rebuild = 1;
   if (i >= d.N) return;
+  if (d.g->pend) flush_atom(d, d.integ->cf, i);
+  d.f[i] = make_float4(0.f, 0.f, 0.f, 0.f);
   const int u = d.id[i];
   const int b = boxid[u];
   const Box& bx = d.box[b];
@@ -2494,18 +2524,9 @@ __global__ void k_load_velocities_keep(Dev d, const double* __restrict__ vin) {
   box_accumulate<1>(ke, b, [&](int bb) { return &d.bst[bb].ke_last; });
 }
 
-// Applies a pending second half-kick (v += dt/2 F/m) before anything changes
-// the forces or the atom order outside a step.
 __global__ void k_flush_pending(Dev d) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (!d.g->pend) return;
-  const double cf = d.integ->cf;
-  if (i < d.N) {
-    const float4 F = d.f[i];
-    d.vx[i] = split_df(join_df(d.vx[i]) + cf * F.x);
-    d.vy[i] = split_df(join_df(d.vy[i]) + cf * F.y);
-    d.vz[i] = split_df(join_df(d.vz[i]) + cf * F.z);
-  }
+  if (d.g->pend && i < d.N) flush_atom(d, d.integ->cf, i);
 }
 
 // Flags every box for a rebuild (new state, parameters, skin or list width).
@@ -2524,26 +2545,21 @@ __host__ __device__ inline int kick_blocks(int n, int threads, int items = 1) {
   return (n + per - 1) / per;
 }
 
-// Zeroes this parity's energy/virial accumulators and (optionally) the forces.
-__global__ void k_prep_force(Dev d, int zero_f) {
-  const int par = (int)(d.g->step & 1ull);
+// The same with the forces (mode 1, 2), a pending half-kick applied with the
+// old ones first (mode 2: the host clears Global::pend after the launch).
+__global__ void k_prep_force(Dev d, int mode) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i == 0) {
-    d.g->n_over = 0;
-    d.g->npairs = 0;
-    d.g->ntrip = 0;
+  prep_box(d, i);
+  if (mode > 0 && i < d.N) {
+    if (mode == 2 && d.g->pend) flush_atom(d, d.integ->cf, i);
+    d.f[i] = make_float4(0.f, 0.f, 0.f, 0.f);
   }
-  if (i < d.nbox)
-    for (int k = 0; k < 8; ++k) d.bst[i].ew[par][k] = 0.0;
-  if (zero_f && i < d.N) d.f[i] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
 // Thermo record from the current accumulators without advancing (forces just
 // evaluated).
-__global__ void k_thermo_snapshot(Dev d) {
-  const Integ I = *d.integ;
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= d.nbox) return;
+__device__ __forceinline__ void thermo_snapshot(const Dev& d, int b) {
+  const Integ& I = *d.integ;
   const int par = (int)(d.g->step & 1ull);
   const BoxState* st = d.bst + b;
   const Box& bx = d.box[b];
@@ -2594,9 +2610,8 @@ __global__ void k_gather_state(Dev d, double* __restrict__ xo, double* __restric
   }
 }
 
-__global__ void k_gather_forces(Dev d, double* __restrict__ fo64, float* __restrict__ fo32) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= d.N) return;
+// Forces to user order.
+__device__ __forceinline__ void gather_force(const Dev& d, int i, double* __restrict__ fo64, float* __restrict__ fo32) {
   const int u = d.id[i];
   const float4 F = d.f[i];
   if (fo64) {
@@ -2625,9 +2640,7 @@ __global__ void k_gather_neighbors(Dev d, int* __restrict__ cnt_out, int* __rest
 // Energies and virial of the latest force evaluation: the parity slot that
 // evaluation wrote (wpar).  After a step the step counter has moved on and
 // its own parity names the slot the next step clears, not this one.
-__global__ void k_energy_out(Dev d, double* e, double* w) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= d.nbox) return;
+__device__ __forceinline__ void energy_out(const Dev& d, int b, double* e, double* w) {
   const int par = d.g->wpar;
   const BoxState* st = d.bst + b;
   if (e) {
@@ -2637,6 +2650,25 @@ __global__ void k_energy_out(Dev d, double* e, double* w) {
   }
   if (w)
     for (int k = 0; k < 6; ++k) w[6 * b + k] = st->ew[par][2 + k];
+}
+
+// What a force call returns, in one launch: the thermo records (snapshot), the
+// forces and the energies and virials, any of them null; nothing after a
+// device error.
+struct ForceOut {
+  double* f64 = nullptr;
+  float* f32 = nullptr;
+  double* e = nullptr;
+  double* w = nullptr;
+};
+__global__ void k_force_out(Dev d, ForceOut o, bool snapshot) {
+  if (*(volatile int*)&d.g->status) return;
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < d.nbox) {
+    if (snapshot) thermo_snapshot(d, i);
+    if (o.e || o.w) energy_out(d, i, o.e, o.w);
+  }
+  if ((o.f64 || o.f32) && i < d.N) gather_force(d, i, o.f64, o.f32);
 }
 
 }  // namespace mw
