@@ -2029,11 +2029,12 @@ __device__ __forceinline__ void bin_item(const Dev& d, int i) {
 // a2: atom i to its sorted slot in the staging arrays: its position with its
 // index (the list is built from these), and, when the box sorts its atoms,
 // the rest of its state.  Otherwise the build position is recorded here.
-__device__ __forceinline__ void scatter_item(const Dev& d, int i) {
+// start: the cells' first slots (d.cell_start, or a shared copy).
+__device__ __forceinline__ void scatter_item(const Dev& d, int i, const int* start) {
   uint4 q = d.q[i];
   const int b = (int)q.w;
   if (!box_flagged(d, b)) return;
-  const int p = d.cell_start[d.cell[i]] + d.rank[i];
+  const int p = start[d.cell[i]] + d.rank[i];
   if ((unsigned)p >= (unsigned)d.N) {  // counts not cleared after an interrupted build: report, write nothing
     set_status(d.g, ST_CELLS);
     d.g->err_index = i;
@@ -2134,7 +2135,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan(Dev d) {
 __global__ void k_scatter(Dev d) {
   if (!d.g->any_rebuild || d.g->status) return;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < d.N) scatter_item(d, i);
+  if (i < d.N) scatter_item(d, i, d.cell_start);
 }
 
 __global__ void k_copyback(Dev d) {

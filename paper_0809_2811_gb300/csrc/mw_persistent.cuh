@@ -181,6 +181,42 @@ __device__ void scan_chunk_offsets(const Dev& d) {
   __syncthreads();
 }
 
+// The scan by every block for itself, into shared memory, for grids whose cell
+// offsets fit there (at most kScanShared cells): no barrier between the counts
+// and the scatter, where the two-level scan has two of 3 us each.  Block b
+// also writes its share of the global offsets, for the list build after the
+// next barrier.  The counts are read with L2 loads and cleared after it.
+constexpr int kScanShared = (int)(sizeof(LegTable) / sizeof(int));
+__device__ void scan_shared(const Dev& d, int* start) {
+  __shared__ int wsum[kPersThreads / 32];
+  const int tid = (int)threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  for (int c = tid; c < d.ncell; c += kPersThreads) start[c] = __ldcg(d.cell_cnt + c);
+  __syncthreads();
+  const int per = (d.ncell + kPersThreads - 1) / kPersThreads | 1;  // odd: threads on different banks
+  const int c0 = min(d.ncell, tid * per), c1 = min(d.ncell, c0 + per);
+  int sum = 0;
+  for (int c = c0; c < c1; ++c) sum += start[c];
+  int incl = sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int t = __shfl_up_sync(kFull, incl, o);
+    if (lane >= o) incl += t;
+  }
+  if (lane == 31) wsum[wid] = incl;
+  __syncthreads();
+  int run = incl - sum;
+  for (int w = 0; w < wid; ++w) run += wsum[w];
+  for (int c = c0; c < c1; ++c) {
+    const int n = start[c];
+    start[c] = run;
+    run += n;
+  }
+  __syncthreads();
+  const int share = (d.ncell + (int)gridDim.x - 1) / (int)gridDim.x, s0 = (int)blockIdx.x * share;
+  for (int c = s0 + tid; c < min(d.ncell, s0 + share); c += kPersThreads) d.cell_start[c] = start[c];
+  if (blockIdx.x == 0 && tid == 0) d.cell_start[d.ncell] = d.N;
+}
+
 // The same two halves as separate kernels, for the per-phase engines (the
 // graph's rebuild body and the host-launched rebuilds): a grid of blocks in
 // place of the single block of k_scan, whose one-block pass over every cell
@@ -234,16 +270,26 @@ __global__ void __launch_bounds__(kPersThreads, kPersBlocksPerSm) k_persistent(c
       for (int i = tid; i < d.N; i += nth) bin_item(d, i);
       phase_mark(d, s, 8);
       if (grid_barrier(g, gen, wait_ns)) return;
-      scan_chunk_local(d);
-      phase_mark(d, s, 9);
-      if (grid_barrier(g, gen, wait_ns)) return;
-      scan_chunk_offsets(d);
-      phase_mark(d, s, 10);
-      if (grid_barrier(g, gen, wait_ns)) return;
-      for (int i = tid; i < d.N; i += nth) scatter_item(d, i);
+      const bool one = d.ncell <= kScanShared;
+      int* const start = one ? reinterpret_cast<int*>(&T) : d.cell_start;
+      if (one) {
+        scan_shared(d, start);
+        phase_mark(d, s, 9);
+        phase_mark(d, s, 10);
+      } else {
+        scan_chunk_local(d);
+        phase_mark(d, s, 9);
+        if (grid_barrier(g, gen, wait_ns)) return;
+        scan_chunk_offsets(d);
+        phase_mark(d, s, 10);
+        if (grid_barrier(g, gen, wait_ns)) return;
+      }
+      for (int i = tid; i < d.N; i += nth) scatter_item(d, i, start);
       phase_mark(d, s, 11);
       if (grid_barrier(g, gen, wait_ns)) return;
       for (int i = tid; i < d.N; i += nth) copyback_item(d, i);
+      if (one)
+        for (int c = tid; c < d.ncell; c += nth) d.cell_cnt[c] = 0;
       phase_mark(d, s, 12);
       {  // the warp's candidate staging slice aliases the leg table (idle until the force phase)
         static_assert(sizeof(LegTable) >= (kPersThreads / 32) * kNSlice * sizeof(float4), "staging slices");
