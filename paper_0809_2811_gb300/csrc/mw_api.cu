@@ -1790,9 +1790,10 @@ std::atomic<unsigned char*> g_na_base[kNaMaxDevices];
 // non-finite value is replaced by 0 and reported (ST_INPUT, the atom in
 // err_index); the host then refuses the call.
 __global__ void k_na_load(Dev d, const double* __restrict__ x) {
+  __shared__ BlockEdges S;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  block_edges(S, d.box, i < d.N ? 0 : -1);
   if (i >= d.N) return;
-  const Box& bx = d.box[0];
   unsigned long long p[3];
   for (int k = 0; k < 3; ++k) {
     double v = x[3 * (size_t)i + k];
@@ -1801,11 +1802,8 @@ __global__ void k_na_load(Dev d, const double* __restrict__ x) {
       d.g->err_index = i;
       v = 0.0;
     }
-    v /= bx.L[k];
-    v -= floor(v);
-    if (v >= 1.0) v -= 1.0;
-    if (v < 0.0) v = 0.0;
-    p[k] = frac64_of(v);
+    int image;
+    p[k] = edge_fraction(S, d.box, 0, k, v, image);
   }
   d.q[i] = make_uint4(q_of(p[0]), q_of(p[1]), q_of(p[2]), 0u);
 }

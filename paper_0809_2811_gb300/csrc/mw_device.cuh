@@ -220,6 +220,99 @@ __device__ __forceinline__ unsigned long long frac64_of(double s) {
   return (t >= 18446744073709551616.0) ? 0ull : __double2ull_rn(t);
 }
 
+// FP64 arithmetic on GB300 runs at 1/64 of the FP32 rate, conversions to and
+// from it included, and a division is ten such instructions: loading a state
+// of 2^20 atoms took 142 us for 22 us of memory traffic, reading it back 62 us.
+// The state's conversions below therefore take integer instructions where the
+// result is the same (61 and 36 us).
+
+// Box fraction of the coordinate x in an edge L, rl = 1 / L: round(x / L 2^64)
+// mod 2^64 (the quotient to its last FP64 bit), and the whole edges below it.
+__device__ __forceinline__ unsigned long long box_fraction(double x, double L, double rl, int& image) {
+  double q = x * rl;
+  q = fma(fma(-q, L, x), rl, q);
+  const unsigned long long u = (unsigned long long)__double_as_longlong(q);
+  const int ex = (int)((u >> 52) & 0x7ffull);
+  const int sh = ex - 1011;  // |q| 2^64 = m 2^sh
+  if (sh > 42) {  // 2^31 edges away or more
+    const double fl = floor(q);
+    image = (int)fl;
+    const double f = q - fl;
+    return f >= 1.0 ? 0ull : frac64_of(f);
+  }
+  const unsigned long long m = (u & 0xfffffffffffffull) | (ex ? 0x10000000000000ull : 0ull);
+  unsigned long long f;
+  int whole = 0;
+  if (sh >= 0) {
+    f = m << sh;
+    if (sh > 11) whole = (int)(m >> (64 - sh));
+  } else if (sh > -64) {  // round to nearest, ties to even
+    const int r = -sh;
+    f = m >> r;
+    const unsigned long long rest = m & ((1ull << r) - 1ull), half = 1ull << (r - 1);
+    f += rest > half || (rest == half && (f & 1ull)) ? 1ull : 0ull;
+  } else {
+    f = 0ull;
+  }
+  if ((long long)u >= 0) {
+    image = whole;
+    return f;
+  }
+  image = -whole - (f ? 1 : 0);
+  return 0ull - f;
+}
+
+// f 2^-64 L of a 64-bit box fraction f, rounded once to FP64: the normalised
+// fraction times L's mantissa, its high half with the rest as a sticky bit.
+__device__ __forceinline__ double fraction_times(unsigned long long f, double L) {
+  if (f == 0ull) return 0.0;
+  const int lz = __clzll((long long)f);
+  const unsigned long long u = (unsigned long long)__double_as_longlong(L);  // (L > 0, normal)
+  const unsigned long long n = f << lz, m = ((u & 0xfffffffffffffull) | 0x10000000000000ull) << 11;
+  const unsigned long long h = __umul64hi(n, m) | (n * m ? 1ull : 0ull);  // f L 2^(1086 + lz - exponent of L)
+  const long long scale = (long long)(u >> 52) - 1086 - lz;
+  return __longlong_as_double(__double_as_longlong(__ull2double_rn(h)) + (scale << 52));
+}
+
+// FP32 to FP64, exact (zero for a subnormal).
+__device__ __forceinline__ double widen(float f) {
+  const uint32_t u = __float_as_uint(f);
+  const uint32_t ex = (u >> 23) & 0xffu;
+  const uint32_t hi = ex == 0u ? 0u : ((ex == 255u ? 2047u : ex + 896u) << 20) | ((u & 0x7fffffu) >> 3);
+  return __hiloint2double((int)((u & 0x80000000u) | hi), ex == 0u ? 0 : (int)(u << 29));
+}
+
+// Reciprocal edges of the boxes of a block's first and last atom, in shared
+// memory (a block of atoms holds one box or two, but for tiny ones).  Called
+// by all threads with their atom's box (b < 0: none; box ids never decrease
+// along atoms); edge() then serves any box.
+struct BlockEdges {
+  double L[2][3], r[2][3];
+  int box[2];
+};
+__device__ __forceinline__ void block_edges(BlockEdges& S, const Box* box, int b) {
+  if (threadIdx.x == 0) {
+    S.box[0] = b;
+    S.box[1] = b;
+  }
+  __syncthreads();
+  if (b >= 0) atomicMax(&S.box[1], b);
+  __syncthreads();
+  if (threadIdx.x < 6 && S.box[0] >= 0) {
+    const int w = (int)threadIdx.x / 3, k = (int)threadIdx.x % 3;
+    const double L = box[S.box[w]].L[k];
+    S.L[w][k] = L;
+    S.r[w][k] = 1.0 / L;
+  }
+  __syncthreads();
+}
+__device__ __forceinline__ unsigned long long edge_fraction(const BlockEdges& S, const Box* box, int b, int k, double x, int& image) {
+  const int w = b == S.box[0] ? 0 : 1;
+  if (b == S.box[w]) return box_fraction(x, S.L[w][k], S.r[w][k], image);
+  const double L = box[b].L[k];
+  return box_fraction(x, L, 1.0 / L, image);
+}
+
 // Exact conversion of an FP32 value to a 64-bit integer with integer
 // operations only (no FP64 or 64-bit conversion instruction): |f| >= 2^23 is
 // an integer already; smaller values round half away from zero; zero and
@@ -241,9 +334,9 @@ __device__ __forceinline__ long long f2ll_exact(float f) {
 // Velocity as hi + lo (FP32 pair) <-> FP64 (set/get state and rare paths only).
 __device__ __forceinline__ float2 split_df(double v) {
   const float hi = (float)v;
-  return make_float2(hi, (float)(v - (double)hi));
+  return make_float2(hi, (float)(v - widen(hi)));
 }
-__device__ __forceinline__ double join_df(float2 v) { return (double)v.x + (double)v.y; }
+__device__ __forceinline__ double join_df(float2 v) { return widen(v.x) + widen(v.y); }
 
 __device__ __forceinline__ float fix_diff(uint32_t a, uint32_t b, float lq) {  // b - a, minimum image
   return __int2float_rn((int)(b - a)) * lq;
@@ -2299,6 +2392,7 @@ __device__ __forceinline__ void prep_box(const Dev& d, int i) {
 // does what k_prep_force does (one launch instead of four: a small box's
 // force call is as long as its launches).
 __global__ void k_load_positions(Dev d, const double* __restrict__ xin, const int* __restrict__ boxid) {
+  __shared__ BlockEdges S;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   prep_box(d, i);
   if (i < d.nbox) {  // every list is stale
@@ -2306,12 +2400,12 @@ __global__ void k_load_positions(Dev d, const double* __restrict__ xin, const in
     d.bst[i].sorted = 0;
   }
   if (i == 0) d.g->any_rebuild = 1;
+  const int u = i < d.N ? d.id[i] : 0;
+  const int b = i < d.N ? boxid[u] : -1;
+  block_edges(S, d.box, b);
   if (i >= d.N) return;
   if (d.g->pend) flush_atom(d, d.integ->cf, i);
   d.f[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-  const int u = d.id[i];
-  const int b = boxid[u];
-  const Box& bx = d.box[b];
   unsigned long long p[3];
   int im[3];
   for (int k = 0; k < 3; ++k) {
@@ -2321,13 +2415,7 @@ __global__ void k_load_positions(Dev d, const double* __restrict__ xin, const in
       d.g->err_index = u;
       v = 0.0;
     }
-    v /= bx.L[k];  // box fraction
-    const double fl = floor(v);
-    im[k] = (int)fl;
-    v -= fl;
-    if (v >= 1.0) v -= 1.0;
-    if (v < 0.0) v = 0.0;
-    p[k] = frac64_of(v);
+    p[k] = edge_fraction(S, d.box, b, k, v, im[k]);
   }
   d.x[i] = p[0]; d.y[i] = p[1]; d.z[i] = p[2];
   if (d.img) d.img[i] = make_int4(im[0], im[1], im[2], 0);
@@ -2365,12 +2453,12 @@ __global__ void k_load_state(Dev d, const double* __restrict__ xin, const double
     d.g->any_rebuild = 1;
     d.g->count_terms = count_terms;
   }
+  __shared__ BlockEdges S;
   float ke[1] = {0.f};
-  int b = -1;
+  const int b = i < d.N ? boxid[i] : -1;
+  block_edges(S, d.box, b);
   if (i < d.N) {
     d.id[i] = i;
-    b = boxid[i];
-    const Box& bx = d.box[b];
     unsigned long long p[3];
     int im[3];
     float vh[3];
@@ -2381,13 +2469,7 @@ __global__ void k_load_state(Dev d, const double* __restrict__ xin, const double
         d.g->err_index = i;
         x = 0.0;
       }
-      double f = x / bx.L[k];  // box fraction
-      const double fl = floor(f);
-      im[k] = (int)fl;
-      f -= fl;
-      if (f >= 1.0) f -= 1.0;
-      if (f < 0.0) f = 0.0;
-      p[k] = frac64_of(f);
+      p[k] = edge_fraction(S, d.box, b, k, x, im[k]);
       double w = vin ? vin[3 * (size_t)i + k] : 0.0;
       if (!isfinite(w)) {
         set_status(d.g, ST_INPUT);
@@ -2422,7 +2504,8 @@ __global__ void k_load_state(Dev d, const double* __restrict__ xin, const double
 // Per-atom parts of k_load_state_keep: slot i's position (fractions, image
 // counts, fixed-point copy, species, zero force, the rebuild flag of its
 // box) and its velocity (FP32 pair; returns its kinetic energy).
-__device__ __forceinline__ void load_keep_position(const Dev& d, const double* __restrict__ xin, int i, float hs2) {
+__device__ __forceinline__ void load_keep_position(const Dev& d, const BlockEdges& S, const double* __restrict__ xin, int i,
+                                                   float hs2) {
   const int u = d.id[i];
   const int b = (int)d.q[i].w;
   const Box& bx = d.box[b];
@@ -2435,13 +2518,7 @@ __device__ __forceinline__ void load_keep_position(const Dev& d, const double* _
       d.g->err_index = u;
       x = 0.0;
     }
-    double f = x / bx.L[k];
-    const double fl = floor(f);
-    im[k] = (int)fl;
-    f -= fl;
-    if (f >= 1.0) f -= 1.0;
-    if (f < 0.0) f = 0.0;
-    p[k] = frac64_of(f);
+    p[k] = edge_fraction(S, d.box, b, k, x, im[k]);
   }
   d.x[i] = p[0];
   d.y[i] = p[1];
@@ -2487,11 +2564,12 @@ __global__ void k_load_state_keep(Dev d, const double* __restrict__ xin, const d
     d.bst[i].Lb = d.box[i].L[0];  // the lists were built in these (unscaled) boxes
   }
   if (i == 0) d.g->count_terms = count_terms;
+  __shared__ BlockEdges S;
   float ke[1] = {0.f};
-  int b = -1;
+  const int b = i < d.N ? (int)d.q[i].w : -1;
+  block_edges(S, d.box, b);
   if (i < d.N) {
-    b = (int)d.q[i].w;
-    load_keep_position(d, xin, i, hs2);
+    load_keep_position(d, S, xin, i, hs2);
     ke[0] = load_keep_velocity(d, I, vin, i);
   }
   box_accumulate<1>(ke, b, [&](int bb) { return &d.bst[bb].ke_last; });
@@ -2510,7 +2588,9 @@ __global__ void k_load_positions_keep(Dev d, const double* __restrict__ xin, int
     d.bst[i].Lb = d.box[i].L[0];
   }
   if (i == 0) d.g->count_terms = count_terms;
-  if (i < d.N) load_keep_position(d, xin, i, hs2);
+  __shared__ BlockEdges S;
+  block_edges(S, d.box, i < d.N ? (int)d.q[i].w : -1);
+  if (i < d.N) load_keep_position(d, S, xin, i, hs2);
 }
 
 __global__ void k_load_velocities_keep(Dev d, const double* __restrict__ vin) {
@@ -2596,18 +2676,24 @@ __global__ void k_gather_state(Dev d, double* __restrict__ xo, double* __restric
   const Box& bx = d.box[d.q[i].w];
   if (xo) {
     constexpr double k2m64 = 5.421010862427522170037264e-20;  // 2^-64
-    const int4 im = unwrap ? d.img[i] : make_int4(0, 0, 0, 0);
-    xo[3 * (size_t)u] = (__ull2double_rn(d.x[i]) * k2m64 + im.x) * bx.L[0];
-    xo[3 * (size_t)u + 1] = (__ull2double_rn(d.y[i]) * k2m64 + im.y) * bx.L[1];
-    xo[3 * (size_t)u + 2] = (__ull2double_rn(d.z[i]) * k2m64 + im.z) * bx.L[2];
+    if (unwrap) {
+      const int4 im = d.img[i];
+      xo[3 * (size_t)u] = (__ull2double_rn(d.x[i]) * k2m64 + im.x) * bx.L[0];
+      xo[3 * (size_t)u + 1] = (__ull2double_rn(d.y[i]) * k2m64 + im.y) * bx.L[1];
+      xo[3 * (size_t)u + 2] = (__ull2double_rn(d.z[i]) * k2m64 + im.z) * bx.L[2];
+    } else {
+      xo[3 * (size_t)u] = fraction_times(d.x[i], bx.L[0]);
+      xo[3 * (size_t)u + 1] = fraction_times(d.y[i], bx.L[1]);
+      xo[3 * (size_t)u + 2] = fraction_times(d.z[i], bx.L[2]);
+    }
   }
   if (vo) {  // pending half-kick and end-of-step thermostat scale applied
     const double s = d.bst[d.q[i].w].s_endc;
     const double cf = d.g->pend ? d.integ->cf : 0.0;
     const float4 F = d.f[i];
-    vo[3 * (size_t)u] = (join_df(d.vx[i]) + cf * F.x) * s;
-    vo[3 * (size_t)u + 1] = (join_df(d.vy[i]) + cf * F.y) * s;
-    vo[3 * (size_t)u + 2] = (join_df(d.vz[i]) + cf * F.z) * s;
+    vo[3 * (size_t)u] = (join_df(d.vx[i]) + cf * widen(F.x)) * s;
+    vo[3 * (size_t)u + 1] = (join_df(d.vy[i]) + cf * widen(F.y)) * s;
+    vo[3 * (size_t)u + 2] = (join_df(d.vz[i]) + cf * widen(F.z)) * s;
   }
 }
 
