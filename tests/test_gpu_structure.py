@@ -114,3 +114,44 @@ def test_structure_limits_and_state(mwlib, orc):
         s.close()
     assert np.allclose(f1, f0, rtol=0, atol=1e-5 * np.abs(f0).max())
     assert abs(e1[0, 0] - e0[0, 0]) <= 1e-6 * (abs(e0[0, 1]) + abs(e0[0, 2]))
+
+
+@pytest.mark.parametrize("n, nc, rho, skin, seed", [(333, 2, 1.0, 1.5, 831), (517, 5, 1.0, 1.5, 832), (700, 16, 1.0, 2.0, 833),
+                                                    (1001, 8, 1.6, 4.0, 834)])  # the last: rows of ~128 entries
+def test_angle_histogram_edges_match_oracle(mwlib, orc, n, nc, rho, skin, seed):
+    """Smallest and largest n_c, last blocks of centres that are not full, and
+    rows longer than the entries a centre's lanes keep."""
+    x, box = I.jittered_box(n, rho, 0.25, seed)
+    x = I.snap_to_grid(x, box)
+    ref, amb, ties = orc.angle_histogram(x, box, nc=nc, nbins=45, tol_deg=0.01)
+    assert ties == 0
+    s = mwlib.System(n, box, skin=skin)
+    try:
+        s.set_state(x)
+        h = s.angle_histogram(nc, 45)[0]
+        assert skin < 4.0 or s.info()["max_count"] > 96
+    finally:
+        s.close()
+    _within_ambiguity(h, ref, amb)
+    assert int(h.sum()) == nc * (nc - 1) * n
+
+
+def test_histograms_of_small_boxes_sharing_a_block(mwlib, orc):
+    """Three and more boxes' centres in one block: their counts reach their own
+    histograms."""
+    xs, boxes = [], []
+    for k in range(9):
+        x, b = (np.array([[1.0, 1.0, 1.0], [3.0 + 0.1 * k, 1.5, 1.2], [2.0, 3.2, 1.0]]), np.array([16.0, 15.0, 14.0]))
+        xs.append(I.snap_to_grid(x, b))
+        boxes.append(b)
+    s = mwlib.System([3] * 9, np.array(boxes))
+    try:
+        s.set_state(np.concatenate(xs))
+        g, a = s.pair_histogram(0.1, 50), s.angle_histogram(2, 30)
+    finally:
+        s.close()
+    for k in range(9):
+        ref, amb = orc.pair_histogram(xs[k], boxes[k], 0.1, 50)
+        _within_ambiguity(g[k], ref, amb)
+        ref, amb, _ = orc.angle_histogram(xs[k], boxes[k], nc=2, nbins=30, tol_deg=0.01)
+        _within_ambiguity(a[k], ref, amb)
