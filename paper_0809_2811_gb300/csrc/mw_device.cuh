@@ -436,7 +436,9 @@ __device__ __forceinline__ bool leg_terms(float r2, const C& c, LegTerms& o, flo
     o.invu = fmaf(v, fmaf(-r, v, 1.0f) - dr * v, v);
     dr = fmaf(r, stretch, dr);
   }
-  if (!(r + dr < c.rc)) return false;
+  // (r itself may still round to the cutoff, or past it, when r + dr does not:
+  // 1/(r - a sig) would then be infinite)
+  if (!(fmaxf(r, r + dr) < c.rc)) return false;
   const float ev = fmaf(-r, v, 1.0f) - dr * v;
   const float xh = r - c.rc;
   const float xl = dr - c.rc_lo;
