@@ -11,13 +11,15 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("sigma", [2.3925, 2.9, 2.0015, 2.75, 3.1, 3.333])
 def test_pairs_at_the_cutoff_are_finite(mwlib, sigma):
     rc = 1.8 * sigma
-    n = 256  # boxes of two atoms, their distances half an ulp apart
-    r = rc * (1.0 + 2.0 ** -25 * (np.arange(n) - 240))
+    n = 2048  # boxes of two atoms, in all directions so that every FP32 squared distance near the cutoff's is met
+    rng = np.random.default_rng(5)
+    u = rng.normal(size=(n, 3))
+    u /= np.linalg.norm(u, axis=1)[:, None]
+    r = rc * (1.0 + 2.0 ** -24 * rng.uniform(-8.0, 2.0, n))
     box = np.tile([40.0, 41.0, 42.0], (n, 1))
     x = np.zeros((2 * n, 3))
-    x[0::2] = [1.0, 2.0, 3.0]
-    x[1::2] = x[0::2]
-    x[1::2, 0] += r
+    x[0::2] = [10.0, 12.0, 13.0]
+    x[1::2] = x[0::2] + r[:, None] * u
     p = mwlib.mw_params_default()
     p.sigma = sigma
     s = mwlib.System([2] * n, box)
