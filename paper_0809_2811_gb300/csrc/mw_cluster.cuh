@@ -74,7 +74,7 @@ __device__ __forceinline__ void clu_st(unsigned a, double v) {
   asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
 }
 
-enum : int { CLU_REBUILD = 1, CLU_STOP = 2 };
+enum : int { CLU_REBUILD = 1, CLU_STOP = 2, CLU_SEEN = 4 };  // (seen: the engine has a status)
 
 struct CluShared {
   Box bx;               // this box, evolved alike by every block (isobaric runs)
@@ -94,7 +94,8 @@ struct CluShared {
 __device__ __forceinline__ void clu_flags(CluShared& S, int ex, int bits, unsigned rank, unsigned size) {
   int all = 0;
   if (__syncthreads_or(bits))
-    all = (__syncthreads_or(bits & CLU_REBUILD) ? CLU_REBUILD : 0) | (__syncthreads_or(bits & CLU_STOP) ? CLU_STOP : 0);
+    all = (__syncthreads_or(bits & CLU_REBUILD) ? CLU_REBUILD : 0) | (__syncthreads_or(bits & CLU_STOP) ? CLU_STOP : 0) |
+          (__syncthreads_or(bits & CLU_SEEN) ? CLU_SEEN : 0);
   if (threadIdx.x < size) clu_st(clu_map(&S.flag[ex & 1][rank], threadIdx.x), all);
 }
 __device__ __forceinline__ int clu_flags_all(const CluShared& S, int ex, unsigned size) {
@@ -231,6 +232,7 @@ __global__ void __launch_bounds__(kCluThreads, 2) k_cluster(const __grid_constan
   Kick1In in{};
   if (on && !mid) in = kick1_load(d, i);
   bool stopped = false;
+  int late = 0;  // flag bits that a quiet step leaves for the next exchange
   int ex = 0;  // flag exchanges so far
   if constexpr (kNpt) {
     // a grid left behind whose report another box's status covered
@@ -247,7 +249,8 @@ __global__ void __launch_bounds__(kCluThreads, 2) k_cluster(const __grid_constan
   }
   while (!stopped && s < A.nsteps) {
     const int par = (int)((A.step0 + (unsigned long long)s) & 1ull);
-    int bits = S.bs.rebuild ? CLU_REBUILD : 0;
+    int bits = (S.bs.rebuild ? CLU_REBUILD : 0) | late;
+    late = 0;
     if (!mid) {
       // a1, a7 first half, a8
       if (on) {
@@ -303,16 +306,32 @@ __global__ void __launch_bounds__(kCluThreads, 2) k_cluster(const __grid_constan
       __syncwarp();
     }
     clu_sync();
+    // Without a thermostat nothing of the next step needs the kinetic energy,
+    // so a step between the run's first (which leaves sig = 0) and its last
+    // ends here: no sums, no barrier, no end_of_step.  Its NaN check and a
+    // status set elsewhere go with the next exchange.  50 steps of 512 atoms:
+    // 730 -> 668 us.
+    const bool quiet = !kNpt && I.kind == TH_NVE && s > 0 && s < A.nsteps - 1 && !(fl & CLU_SEEN);
+    if (quiet) {
+      if (tid == 0 && *(volatile int*)&d.g->status) late = CLU_SEEN;
+      if (on) {
+        in = kick1_load(d, i);
+        if (!(kick2_energy(I, in.F, in.v) < 1e30f)) {
+          set_status_nan(d.g);
+          d.g->err_index = i;
+          late |= CLU_STOP;
+        }
+      }
+      mid = false;
+      pend = 1;
+      ++s;
+      continue;
+    }
     // a7 second half: the kinetic energy of v + a, and the next kick1's inputs
     float ke = 0.f;
     if (on) {
       in = kick1_load(d, i);
-      const float Fc[3] = {in.F.x, in.F.y, in.F.z};
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        const float u = fmaf(I.cf_f, Fc[c], in.v[c].x) + in.v[c].y;
-        ke += (float)I.ke_fac * u * u;
-      }
+      ke = kick2_energy(I, in.F, in.v);
     }
     const bool nan = !(ke < 1e30f);
     if (nan) {

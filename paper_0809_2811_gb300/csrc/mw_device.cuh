@@ -517,6 +517,11 @@ __device__ __forceinline__ int cell_of(const uint4& q, const Box& bx) {
 }
 
 __device__ __forceinline__ void set_status(Global* g, int st) { atomicCAS(&g->status, 0, st); }
+// A NaN found together with the next kick1's checks: its status stands over
+// the runaway velocity that the same NaN makes there.
+__device__ __forceinline__ void set_status_nan(Global* g) {
+  if (atomicCAS(&g->status, 0, (int)ST_NAN) == ST_LOST) atomicCAS(&g->status, (int)ST_LOST, (int)ST_NAN);
+}
 
 // Arrival on a block counter, acq_rel at gpu scope: after a __syncthreads it
 // publishes the whole block's writes (the barrier orders them before thread
@@ -1021,8 +1026,21 @@ __device__ __forceinline__ void kick1_apply(const Dev& d, const Integ& I, const 
   moved = dd > (kNpt ? bx.hs2 : I.half_skin2);
 }
 
+// The kinetic energy of v + a (FP32 per component and per atom).
+__device__ __forceinline__ float kick2_energy(const Integ& I, const float4& F, const float2 (&v)[3]) {
+  const float Fc[3] = {F.x, F.y, F.z};
+  float ke = 0.f;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const float u = fmaf(I.cf_f, Fc[c], v[c].x) + v[c].y;
+    ke += (float)I.ke_fac * u * u;
+  }
+  return ke;
+}
+
+// late: the step before left its NaN check to this one.
 template <bool kNpt>
-__device__ __forceinline__ void kick1_atom(const Dev& d, const Integ& I, int i, int par, int pend) {
+__device__ __forceinline__ void kick1_atom(const Dev& d, const Integ& I, int i, int par, int pend, bool late = false) {
   // every load first (nothing here is written by another atom's thread);
   // the fixed-point copy is read only for its box (one box: box 0)
   const int b = d.nbox == 1 ? 0 : (int)d.q[i].w;
@@ -1044,6 +1062,10 @@ __device__ __forceinline__ void kick1_atom(const Dev& d, const Integ& I, int i, 
     set_status(d.g, ST_LOST);
     d.g->err_index = i;
   }
+  if (late && !(kick2_energy(I, in.F, in.v) < 1e30f)) {
+    set_status_nan(d.g);
+    d.g->err_index = i;
+  }
 }
 
 // a7 (second half): the kinetic energy of atom i's v + a (FP32 per
@@ -1056,13 +1078,7 @@ __device__ __forceinline__ float kick2_atom(const Dev& d, const Integ& I, int i,
   b = d.nbox == 1 ? 0 : (int)d.q[i].w;
   const float4 F = d.f[i];
   const float2 v[3] = {d.vx[i], d.vy[i], d.vz[i]};
-  const float Fc[3] = {F.x, F.y, F.z};
-  float ke = 0.f;
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    const float u = fmaf(I.cf_f, Fc[c], v[c].x) + v[c].y;
-    ke += (float)I.ke_fac * u * u;
-  }
+  const float ke = kick2_energy(I, F, v);
   if (!(ke < 1e30f)) {
     set_status(d.g, ST_NAN);
     d.g->err_index = i;
