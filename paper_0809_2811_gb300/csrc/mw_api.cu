@@ -1133,7 +1133,7 @@ mw_status create_common(mw_system** out, int nbox, const int* n, const double* b
       (st = dalloc(s, &d.tq, N)) != MW_OK || (st = dalloc(s, &d.f, N)) != MW_OK ||
       (st = dalloc(s, &d.id, N)) != MW_OK || (st = dalloc(s, &d.tid, N)) != MW_OK ||
       (st = dalloc(s, &d.cell, N)) != MW_OK || (st = dalloc(s, &d.rank, N)) != MW_OK ||
-      (st = dalloc(s, &d.nbr_cnt, N)) != MW_OK || (st = dalloc(s, &d.over, N)) != MW_OK ||
+      (st = dalloc(s, &d.nbr_cnt, N)) != MW_OK || (st = dalloc(s, &d.bar, 2 * kBarStride)) != MW_OK ||
       (st = dalloc(s, &d.stage, 3 * N)) != MW_OK || (st = dalloc(s, &d.stage2, 3 * N)) != MW_OK ||
       (st = dalloc(s, &s->boxid, N)) != MW_OK || (st = dalloc(s, &s->eout, 9 * (size_t)nbox)) != MW_OK ||
       (st = dalloc(s, &d.chunk, 4096)) != MW_OK)
@@ -1764,8 +1764,7 @@ constexpr size_t kNaCell = kNaF + na_align(sizeof(float4) * MW_NOALLOC_MAX_ATOMS
 constexpr size_t kNaRank = kNaCell + na_align(sizeof(int) * MW_NOALLOC_MAX_ATOMS);
 constexpr size_t kNaTid = kNaRank + na_align(sizeof(int) * MW_NOALLOC_MAX_ATOMS);
 constexpr size_t kNaCnt = kNaTid + na_align(sizeof(int) * MW_NOALLOC_MAX_ATOMS);
-constexpr size_t kNaOver = kNaCnt + na_align(sizeof(int) * MW_NOALLOC_MAX_ATOMS);
-constexpr size_t kNaNbr = kNaOver + na_align(sizeof(int) * MW_NOALLOC_MAX_ATOMS);
+constexpr size_t kNaNbr = kNaCnt + na_align(sizeof(int) * MW_NOALLOC_MAX_ATOMS);
 constexpr size_t kNaCellCnt = kNaNbr + na_align(sizeof(int) * (size_t)MW_NOALLOC_MAX_ATOMS * MW_NOALLOC_MAX_WIDTH);
 constexpr size_t kNaCellStart = kNaCellCnt + na_align(sizeof(int) * MW_NOALLOC_MAX_CELLS);
 constexpr size_t kNaCellBox = kNaCellStart + na_align(sizeof(int) * (MW_NOALLOC_MAX_CELLS + 1));
@@ -1930,7 +1929,6 @@ extern "C" mw_status mw_energy_forces_noalloc(int n, const double box[3], const 
   d.rank = (int*)(base + kNaRank);
   d.tid = (int*)(base + kNaTid);
   d.nbr_cnt = (int*)(base + kNaCnt);
-  d.over = (int*)(base + kNaOver);
   d.nbr = (int*)(base + kNaNbr);
   d.cell_cnt = (int*)(base + kNaCellCnt);
   d.cell_start = (int*)(base + kNaCellStart);

@@ -3,8 +3,8 @@
 //
 // The steps of a small box are a chain of short phases (kick1 | list | force |
 // kick2 + thermostat), each a microsecond or so of work, and a grid-wide
-// barrier through L2 costs 1.6 to 3.5 us (5.6 to 9 with 760 blocks), five more
-// on a rebuild.  Boxes of a batch do not depend on one another, so nothing
+// barrier through L2 costs 1.1 to 1.6 us beside the wait for the slowest
+// block.  Boxes of a batch do not depend on one another, so nothing
 // needs a grid-wide barrier: the hardware cluster barrier orders a box's
 // phases, small sums and flags travel through distributed shared memory, the
 // thermostat is evaluated by every block for itself, and a box rebuilds its

@@ -99,8 +99,7 @@ struct Global {
   unsigned done1;           // last-block counter of k_kick1 (graph condition)
   long long rebuild_steps;  // steps (or force calls) that rebuilt at least one box
   int pend;                 // 1: velocities lack the second half-kick of the last step
-  unsigned bar_count, bar_gen;  // persistent engine grid barrier
-  int bar_stat[2];              // status snapshot taken at each barrier release
+  int pad_bar[4];           // (unused: checkpoints hold this struct)
   long long npairs, ntrip;  // leg / triplet counts of the last force call (if counting)
   int count_terms;
   int n_over;               // centres routed to the overflow path
@@ -170,7 +169,7 @@ struct Dev {
   int *cell_cnt, *cell_start;
   int* cell_box;      // box of each global cell
   int *nbr, *nbr_cnt;
-  int* over;          // overflow centre list
+  unsigned long long* bar;  // grid barrier of the persistent engine: two counters, kBarStride apart
   int* chunk;         // per-block cell totals of the persistent engine's scan
   int chunk_cap;
   const Box* box;
@@ -516,10 +515,20 @@ __device__ __forceinline__ int cell_of(const uint4& q, const Box& bx) {
   return bx.cell_off + cx + bx.nc[0] * (cy + bx.nc[1] * cz);
 }
 
-__device__ __forceinline__ void set_status(Global* g, int st) { atomicCAS(&g->status, 0, st); }
+// The block's own error flag, for the engine whose barriers carry it (the
+// other kernels neither clear nor read it).
+__device__ __forceinline__ int& block_error() {
+  __shared__ int s_error;
+  return s_error;
+}
+__device__ __forceinline__ void set_status(Global* g, int st) {
+  block_error() = 1;
+  atomicCAS(&g->status, 0, st);
+}
 // A NaN found together with the next kick1's checks: its status stands over
 // the runaway velocity that the same NaN makes there.
 __device__ __forceinline__ void set_status_nan(Global* g) {
+  block_error() = 1;
   if (atomicCAS(&g->status, 0, (int)ST_NAN) == ST_LOST) atomicCAS(&g->status, (int)ST_LOST, (int)ST_NAN);
 }
 
@@ -531,14 +540,6 @@ __device__ __forceinline__ unsigned bar_arrive(unsigned* p) {
   unsigned old;
   asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(old) : "l"(p) : "memory");
   return old + 1u;
-}
-__device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
-  unsigned v;
-  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
-__device__ __forceinline__ void st_release(unsigned* p, unsigned v) {
-  asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
 // Rebuilds are per box.  On a rebuild step every atom is binned and the scan
