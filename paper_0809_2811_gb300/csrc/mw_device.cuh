@@ -1039,16 +1039,18 @@ __device__ __forceinline__ float kick2_energy(const Integ& I, const float4& F, c
   return ke;
 }
 
-// late: the step before left its NaN check to this one.
+// boxes, states: d.box and d.bst, or a block's own copies of the fields read
+// here.  late: the step before left its NaN check to this one.
 template <bool kNpt>
-__device__ __forceinline__ void kick1_atom(const Dev& d, const Integ& I, int i, int par, int pend, bool late = false) {
+__device__ __forceinline__ void kick1_atom(const Dev& d, const Integ& I, int i, int par, int pend, const Box* boxes,
+                                           const BoxState* states, bool late) {
   // every load first (nothing here is written by another atom's thread);
   // the fixed-point copy is read only for its box (one box: box 0)
   const int b = d.nbox == 1 ? 0 : (int)d.q[i].w;
   const Kick1In in = kick1_load(d, i);
-  const Box& bx = d.box[b];
+  const Box& bx = boxes[b];
   bool moved, lost;
-  kick1_apply<kNpt>(d, I, bx, d.bst[b].sig, i, b, pend, in, moved, lost);
+  kick1_apply<kNpt>(d, I, bx, states[b].sig, i, b, pend, in, moved, lost);
   if (i == bx.off) {  // this step's accumulators start from zero
     BoxState* sw = d.bst + b;
     sw->ke_acc[par] = 0.0;
@@ -2113,7 +2115,7 @@ __global__ void __launch_bounds__(kKThreads, 6) k_kick1(Dev d, cudaGraphConditio
   const int pend = d.g->pend;
   if (blockIdx.x == 0 && threadIdx.x == 0) d.g->n_over = 0;
   const int i = (int)(blockIdx.x * blockDim.x + threadIdx.x);
-  if (i < d.N) kick1_atom<kNpt>(d, I, i, par, pend);
+  if (i < d.N) kick1_atom<kNpt>(d, I, i, par, pend, d.box, d.bst, false);
   if constexpr (kCond || kNpt) {
     __shared__ bool last;
     __syncthreads();
