@@ -58,6 +58,7 @@ __device__ __forceinline__ unsigned long long globaltimer_ns() {
 // Waits are bounded by limit_ns of wall time (0: given up at once); a block
 // that gives up sets ST_TIMEOUT and leaves, and so do the others in time.
 constexpr int kBarStride = 16;  // 128 bytes
+constexpr int kBarPrior = 1;    // beside the first counter: non-zero if an earlier launch of the run met an error
 struct GridBar {  // per block, in shared memory
   unsigned long long limit_ns;
   unsigned passed;     // barriers passed in this launch
@@ -276,6 +277,7 @@ __global__ void __launch_bounds__(kPersThreads, kPersBlocksPerSm) k_persistent(c
   __shared__ Box s_box[kNpt ? 1 : kOwnBoxes];
   __shared__ BoxState s_bst[kNpt ? 1 : kOwnBoxes];
   Global* g = d.g;
+  if (d.bar[kBarPrior]) return;
   const bool own = !kNpt && d.nbox <= kOwnBoxes;
   if (own && (int)threadIdx.x < d.nbox) {
     s_box[threadIdx.x] = d.box[threadIdx.x];

@@ -40,3 +40,25 @@ def test_boxes_match_oracle(mwlib, orc, nbox, kind):
         assert th[k]["pe"] == pytest.approx(tho[-1, 0], rel=3e-6)
         assert th[k]["ke"] == pytest.approx(tho[-1, 3], rel=1e-5)
         assert th[k]["xi"] == pytest.approx(st[0], rel=1e-4, abs=1e-9)
+
+
+@pytest.mark.parametrize("steps", [100000, 100001])  # one launch; two
+def test_long_asynchronous_runs(mwlib, steps):
+    """Three atoms out of each other's reach, with one velocity: a straight line."""
+    box = np.array([40.0, 41.0, 42.0])
+    x = np.array([[1.0, 2.0, 3.0], [11.0, 2.0, 3.0], [1.0, 22.0, 3.0]])
+    v = np.tile([2.0e-4, 0.0, -1.0e-4], (3, 1))
+    s = mwlib.System(3, box)
+    try:
+        s.set_engine(mwlib.MW_ENGINE_PERSISTENT)
+        s.set_state(x, v)
+        mwlib.mw_step_async(s.h, mwlib.make_integrator(10.0, mwlib.MW_NVE, 300.0, 1000.0), steps)
+        mwlib.mw_sync(s.h)
+        assert s.thermo()[0]["step"] == steps
+        xg, vg = s.get_state()
+    finally:
+        s.close()
+    d = xg - (x + v * 10.0 * steps)
+    # each step's move is rounded to FP32 (relative 6e-8): below 200 A * 6e-8
+    assert np.abs(d - box * np.rint(d / box)).max() < 2e-5
+    assert np.abs(vg - v).max() < 1e-12
