@@ -1537,16 +1537,19 @@ mw_status mw_forces_async(mw_system* s) {
 }
 
 // The engine of MW_ENGINE_AUTO where no autotuner has chosen: the persistent
-// one, above 150000 atoms the graph engine.  The grid-wide kernel runs every
-// phase at the force phase's 20 warps an SM; from about 10^5 atoms on the
-// separate kernels' 32 are worth more than the launches between them (20
-// steps, skin 1 A: 65536 atoms 1065 us persistent, 1194 graph; 100000 1424 /
-// 1419; 200000 2418 / 2356; 400000 4778 / 4447; 256 uneven boxes of 1.16 10^6
-// atoms 11808 / 10455).  Isobaric runs stay: the persistent tail is quicker
-// (64000 atoms 2024 / 2753).
+// one, and the graph engine above 200000 atoms (150000 in batches whose
+// thermostats the last block evaluates).  The grid-wide kernel runs every
+// phase at the force phase's 20 warps an SM; for large systems the separate
+// kernels' 32 are worth more than the launches between them.  20 steps, skin
+// 1 A, us, persistent / graph: 65536 atoms 932 / 1172, 150000 1888 / 1934,
+// 200000 2232 / 2280, 230000 2743 / 2730; without a thermostat 150000 1796 /
+// 1925, 230000 2632 / 2737; 38 boxes of 4000 2325 / 2262, 50 2728 / 2653; 256
+// uneven boxes of 1.16 10^6 atoms 11808 / 10455.  Isobaric runs stay: the
+// persistent tail is quicker (64000 atoms 1826 / 2696).
 static int auto_engine(const mw_system* s) {
   if (s->tuned_engine >= 0) return s->tuned_engine;
-  return s->N > 150000 && s->integ.kind != TH_NPT ? MW_ENGINE_GRAPH : MW_ENGINE_PERSISTENT;
+  const int most = s->nbox <= kOwnBoxes ? 200000 : 150000;
+  return s->N > most && s->integ.kind != TH_NPT ? MW_ENGINE_GRAPH : MW_ENGINE_PERSISTENT;
 }
 
 mw_status mw_step(mw_system* s, const mw_integrator* integ, int nsteps, mw_thermo* last) {

@@ -8,11 +8,11 @@
 // Dynamics: velocity Verlet with Berendsen or Nose-Hoover (Sec. II.B).
 //
 // Layout (all boxes concatenated box-major, atoms sorted by cell inside each
-// box at every neighbour-list rebuild):
-//   x,y,z            FP64 master positions as fractions of the box edge, [0, 1)
-//   vx,vy,vz         FP64 master velocities (A/fs); between steps they lack the
-//                    second half-kick of the last step (Global::pend), which
-//                    the next kick1 folds into its own
+// box at every eighth neighbour-list rebuild):
+//   x,y,z            master positions as 64-bit fractions of the box edge
+//   vx,vy,vz         master velocities (A/fs) as FP32 sums hi + lo; between
+//                    steps they lack the second half-kick of the last step
+//                    (Global::pend), which the next kick1 folds into its own
 //   q                uint4 {qx, qy, qz, box}: position as a 32-bit fraction of
 //                    the box edge; the minimum-image difference of two atoms
 //                    is the wrapping int32 difference, converted once to FP32
@@ -102,7 +102,7 @@ struct Global {
   int pad_bar[4];           // (unused: checkpoints hold this struct)
   long long npairs, ntrip;  // leg / triplet counts of the last force call (if counting)
   int count_terms;
-  int n_over;               // centres routed to the overflow path
+  int pad_over;             // (unused)
   int err_index;
   int pad_;
 };
@@ -202,10 +202,6 @@ constexpr int kPhaseMarks = 16;  // 14 used
 
 // ---------------------------------------------------------------------------
 // small helpers
-
-__device__ __forceinline__ uint32_t to_fixed(double x, double qs) {
-  return (uint32_t)(unsigned long long)__double2ll_rn(x * qs);
-}
 
 // 32-bit fixed-point coordinate of a 64-bit box fraction: round(s / 2^32)
 // mod 2^32 (a fraction within half a unit of 1 wraps to 0).
@@ -2113,7 +2109,6 @@ __global__ void __launch_bounds__(kKThreads, 6) k_kick1(Dev d, cudaGraphConditio
   const Integ I = *d.integ;
   const int par = (int)(d.g->step & 1ull);
   const int pend = d.g->pend;
-  if (blockIdx.x == 0 && threadIdx.x == 0) d.g->n_over = 0;
   const int i = (int)(blockIdx.x * blockDim.x + threadIdx.x);
   if (i < d.N) kick1_atom<kNpt>(d, I, i, par, pend, d.box, d.bst, false);
   if constexpr (kCond || kNpt) {
@@ -2400,7 +2395,6 @@ __device__ __forceinline__ void flush_atom(const Dev& d, double cf, int i) {
 __device__ __forceinline__ void prep_box(const Dev& d, int i) {
   const int par = (int)(d.g->step & 1ull);
   if (i == 0) {
-    d.g->n_over = 0;
     d.g->npairs = 0;
     d.g->ntrip = 0;
   }

@@ -1,8 +1,8 @@
 // mw_persistent.cuh -- persistent engine: one cooperative launch advances
 // every box nsteps MD steps, with grid-wide barriers between the phases of
-// mw_device.cuh (kick1 | [bin | scan | scan | scatter | copy + neighbour
-// list] | force | kick2 + thermostat in the last block to arrive).  All blocks are
-// co-resident (cooperative launch), every barrier wait is bounded in wall
+// mw_device.cuh (kick1 | [bin | scan | scatter | copy + neighbour list] |
+// force | kick2, then the thermostats: by every block, or in larger batches by
+// the last block to arrive).  All blocks are co-resident (cooperative launch), every barrier wait is bounded in wall
 // time, and each barrier's counter carries the blocks' error flags, so that
 // all blocks take the same decision to stop.  Data written in one phase is
 // read by other blocks in a later phase of the same launch, so those reads
@@ -304,7 +304,6 @@ __global__ void __launch_bounds__(kPersThreads, kPersBlocksPerSm) k_persistent(c
     const int par = (int)(step & 1ull);
     phase_mark(d, s, 0);
     // a1 + a7 first half, a8 displacement check
-    if (tid == 0) g->n_over = 0;
     if (quiet && tid == 0) g->step = step;  // (the step before left that, and its NaN check, to this one)
     for (int i = tid; i < d.N; i += nth) kick1_atom<kNpt>(d, I, i, par, pend, boxes, states, quiet);
     pend = 1;
