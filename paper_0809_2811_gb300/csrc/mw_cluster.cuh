@@ -220,7 +220,9 @@ __global__ void __launch_bounds__(kCluThreads, 2) k_cluster(const __grid_constan
   int s = A.prog[b];
   bool mid = A.mid[b] != 0;
   int pend = s > 0 ? 1 : d.g->pend;
-  __syncthreads();
+  // Every block of the cluster has started and has its copies: from here on
+  // others store into its shared memory, and rank 0 writes the box's globals.
+  clu_sync();
   const Integ& I = S.I;
   const int off = S.bx.off, n = S.bx.n;
   const int per = (n + (int)size - 1) / (int)size;  // atoms of a block
