@@ -340,7 +340,7 @@ mw_status mw_get_box(mw_system* s, double* box);
  *   dL_dtheta[nbox*3] (host doubles, may be NULL) = sum_i w_i . dF_i/d(lambda, epsilon, sigma)
  *   per box.
  * The forward leg and triplet quantities are recomputed, not stored.
- * The neighbour list must be current (call mw_energy_forces first). */
+ * The neighbour list is built first if it is stale. */
 mw_status mw_energy_forces_vjp(mw_system* s, const float* dL_dF_dev, float* dL_dx_dev, double* dL_dtheta);
 
 /* Selects the engine mw_step uses (mw_engine).  MW_ENGINE_PLAIN is refused

@@ -75,6 +75,10 @@ struct mw_system {
   bool v_pending = false;
   bool own_stream = false;
   bool list_built = false;
+  // some rows were given up (a new row array, a restored checkpoint) and not
+  // built since, though the forces may still be valid: whatever reads the rows
+  // outside a step builds them first (ensure_rows)
+  bool rows_stale = false;
   // the atom order and neighbour lists are current for the geometry and
   // parameters (set by a completed force call; cleared by anything that
   // flags every box for a rebuild, by a failed run, by isobaric steps):
@@ -125,6 +129,7 @@ struct mw_system {
   // its cluster form: one buffer for the box order and the per-box progress
   int* clu_order = nullptr;
   bool clu_resume = false;  // the next launch goes on with boxes that stopped on their own steps
+  bool clu_left = false;    // the last run ended with a box flagged for a build
   std::vector<int> cell_box_host;
   std::vector<void*> allocs;
   // pinned host staging for the small device-to-host reads (the Global
@@ -313,6 +318,8 @@ mw_status alloc_nbr(mw_system* s, int W) {
   MW_CUDA(cudaMemsetAsync(s->d.nbr, 0, sizeof(int) * (size_t)W * s->N, s->stream));
   s->W = s->d.W = W;
   s->list_built = false;
+  s->rows_stale = true;
+  s->lists_current = false;
   s->order_ok = false;
   s->graph_dirty = true;
   return MW_OK;
@@ -658,6 +665,7 @@ mw_status ensure_forces(mw_system* s, const ForceOut* out = nullptr, bool prepar
     if (g.status) return status_error(g);
     s->forces_valid = true;
     s->list_built = true;
+    s->rows_stale = false;
     s->order_ok = s->integ.kind != TH_NPT;
     s->record_pending = false;  // the snapshot is the newest record
     s->g_known = g;
@@ -721,6 +729,24 @@ mw_status regrid(mw_system* s) {
   s->regrids += 1;
   s->boxes_stale = true;  // the run goes on scaling the boxes
   return MW_OK;
+}
+
+// Forces and whole rows at the current positions: a force call of its own if
+// rows are missing.  (The pending half-kick is applied with the old forces.)
+mw_status ensure_rows(mw_system* s) {
+  if (s->rows_stale && s->state_set && s->forces_valid) {
+    mw_status st;
+    Global g;
+    if ((st = read_global(s, &g)) != MW_OK) return st;
+    if (g.status == ST_GRID) {  // left at a step boundary: the cells are laid out again first
+      if ((st = regrid(s)) != MW_OK) return st;
+      s->graph_dirty = true;
+    } else if (g.status) {
+      return status_error(g);
+    }
+    s->forces_valid = false;
+  }
+  return ensure_forces(s);
 }
 
 // The start-of-step thermostat half is normally computed at the end of the
@@ -1455,6 +1481,7 @@ mw_status mw_build_neighbors(mw_system* s, int* max_count_out) {
     MW_CUDA(cudaStreamSynchronize(s->stream));
     s->forces_valid = false;  // atoms were re-sorted; stored forces no longer line up
     s->list_built = true;
+    s->rows_stale = false;
     if (max_count_out) *max_count_out = g.max_count;
     return MW_OK;
   }
@@ -1467,6 +1494,7 @@ mw_status mw_get_neighbors(mw_system* s, int* counts, int* nbr, int width) {
   int* dc;
   int* dn;
   mw_status st;
+  if (s->rows_stale && (st = ensure_rows(s)) != MW_OK) return st;
   if ((st = dalloc(s, &dc, s->N)) != MW_OK) return st;
   if ((st = dalloc(s, &dn, (size_t)s->N * width)) != MW_OK) {
     dfree(s, dc);
@@ -1529,7 +1557,7 @@ mw_status mw_energy_forces_dev(mw_system* s, const double* x_dev, float* f_dev, 
 mw_status mw_forces_async(mw_system* s) {
   if (!s) return fail(MW_EINVAL, "system is NULL");
   mw_status st;
-  if ((st = ensure_forces(s)) != MW_OK) return st;
+  if ((st = ensure_rows(s)) != MW_OK) return st;
   k_prep_force<<<div_up(std::max(s->N, s->nbox), kThreads), kThreads, 0, s->stream>>>(s->d, 1);
   launch_force(s);
   MW_CUDA(cudaGetLastError());
@@ -1567,6 +1595,7 @@ mw_status mw_step(mw_system* s, const mw_integrator* integ, int nsteps, mw_therm
     if (eng == MW_ENGINE_PERSISTENT && !persistent_available(s)) eng = MW_ENGINE_GRAPH;
     s->engine_used = eng;
     CluConfig clu;
+    s->clu_left = false;
     st = eng == MW_ENGINE_PERSISTENT
              ? (cluster_config(s, nsteps, &clu) ? run_cluster_engine(s, clu, nsteps, last, &fetched)
                                         : run_persistent_engine(s, nsteps, last, &fetched))
@@ -1578,6 +1607,9 @@ mw_status mw_step(mw_system* s, const mw_integrator* integ, int nsteps, mw_therm
       return st;
     }
     s->list_built = true;
+    // the steps built every row, but for boxes that had finished theirs
+    // when the cluster form grew the rows: those are flagged still
+    s->rows_stale = s->rows_stale && eng == MW_ENGINE_PERSISTENT && s->clu_left;
   }
   if (last && !fetched) return mw_get_thermo(s, last);
   return MW_OK;
@@ -1597,6 +1629,7 @@ mw_status mw_step_async(mw_system* s, const mw_integrator* integ, int nsteps) {
   s->engine_used = eng;
   if ((st = prime_thermostat(s)) != MW_OK) return st;
   s->record_pending = true;
+  s->rows_stale = false;  // (the first step builds them)
   if (eng == MW_ENGINE_PERSISTENT) return enqueue_persistent(s, nsteps);
   if (eng == MW_ENGINE_PLAIN) return launch_plain_steps(s, nsteps);
   if (s->graph_dirty || !s->graph1) {
