@@ -629,8 +629,11 @@ mw_status ensure_forces(mw_system* s, const ForceOut* out = nullptr, bool prepar
     if (!out) return MW_OK;
     k_force_out<<<go, kThreads, 0, s->stream>>>(s->d, o, false);
     MW_CUDA(cudaGetLastError());
-    MW_CUDA(cudaStreamSynchronize(s->stream));
-    return MW_OK;
+    Global g;
+    if ((st = read_global(s, &g)) != MW_OK) return st;
+    if (g.status == ST_OK || g.status == ST_GRID) return MW_OK;
+    s->order_ok = false;  // an asynchronous run failed: its state is not one to report forces of
+    return status_error(g);
   }
   if ((st = set_func_attrs()) != MW_OK) return st;
   // a state just set in the kept order may have told that no list is stale

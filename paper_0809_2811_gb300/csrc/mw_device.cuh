@@ -2754,9 +2754,12 @@ __device__ __forceinline__ void energy_out(const Dev& d, int b, double* e, doubl
     for (int k = 0; k < 6; ++k) w[6 * b + k] = st->ew[par][2 + k];
 }
 
-// What a force call returns, in one launch: the thermo records (snapshot), the
-// forces and the energies and virials, any of them null; nothing after a
-// device error.
+// What a force call returns, in one launch: the forces and the energies and
+// virials, any of them null, and the thermo records of a force call just made
+// (snapshot).  Nothing after a device error: a fresh call has evaluated
+// nothing then, and of earlier forces the host reports the error.  An isobaric
+// box that left its cell grid (ST_GRID) did so at a step boundary, whose
+// forces are valid.
 struct ForceOut {
   double* f64 = nullptr;
   float* f32 = nullptr;
@@ -2764,7 +2767,8 @@ struct ForceOut {
   double* w = nullptr;
 };
 __global__ void k_force_out(Dev d, ForceOut o, bool snapshot) {
-  if (*(volatile int*)&d.g->status) return;
+  const int st = *(volatile int*)&d.g->status;
+  if (st && (snapshot || st != ST_GRID)) return;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < d.nbox) {
     if (snapshot) thermo_snapshot(d, i);
