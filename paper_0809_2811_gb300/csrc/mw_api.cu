@@ -156,7 +156,7 @@ struct Range {
 mw_status persistent_func_attrs();
 bool persistent_available(mw_system* s);
 mw_status run_persistent_engine(mw_system* s, int nsteps, mw_thermo* last, bool* fetched);
-mw_status enqueue_persistent(mw_system* s, int nsteps);
+mw_status enqueue_persistent(mw_system* s, int nsteps, bool checked);
 mw_status adjoint_alloc(mw_system* s);
 mw_status prime_thermostat(mw_system* s);
 
@@ -1632,8 +1632,7 @@ mw_status mw_step_async(mw_system* s, const mw_integrator* integ, int nsteps) {
   s->engine_used = eng;
   if ((st = prime_thermostat(s)) != MW_OK) return st;
   s->record_pending = true;
-  s->rows_stale = false;  // (the first step builds them)
-  if (eng == MW_ENGINE_PERSISTENT) return enqueue_persistent(s, nsteps);
+  if (eng == MW_ENGINE_PERSISTENT) return enqueue_persistent(s, nsteps, false);
   if (eng == MW_ENGINE_PLAIN) return launch_plain_steps(s, nsteps);
   if (s->graph_dirty || !s->graph1) {
     if ((st = capture_graphs(s, 16)) != MW_OK) return st;

@@ -58,7 +58,7 @@ __device__ __forceinline__ unsigned long long globaltimer_ns() {
 // Waits are bounded by limit_ns of wall time (0: given up at once); a block
 // that gives up sets ST_TIMEOUT and leaves, and so do the others in time.
 constexpr int kBarStride = 16;  // 128 bytes
-constexpr int kBarPrior = 1;    // beside the first counter: non-zero if an earlier launch of the run met an error
+constexpr int kBarPrior = 1;    // beside the first counter: non-zero if the work before this launch met an error
 struct GridBar {  // per block, in shared memory
   unsigned long long limit_ns;
   unsigned passed;     // barriers passed in this launch
