@@ -354,13 +354,13 @@ __global__ void __launch_bounds__(kCluThreads, 2) k_cluster(const __grid_constan
     if (lane == 0) S.warp[wid][8] = ke;
     const int st0 = tid == 0 ? *(volatile int*)&d.g->status : 0;  // an error of another box, or of the overflow path
     clu_flags(S, ++ex, (nan || st0) ? CLU_STOP : 0, rank, size);
-    // this block's sums to every block: FP32 within a warp (kinetic energy:
-    // within the block), FP64 above
+    // this block's sums to every block: FP32 within a warp, FP64 above
     if (wid == 0) {
-      float v = lane < nwarp ? S.warp[lane][8] : 0.f;
+      double v = lane < nwarp ? (double)S.warp[lane][8] : 0.0;
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
-      if (lane < (int)size) clu_st(clu_map(&S.sum[rank][8], lane), (double)v);
+      for (int o = nwarp / 2; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
+      static_assert(kCluMax <= nwarp, "every lane that stores the sum has it");
+      if (lane < (int)size) clu_st(clu_map(&S.sum[rank][8], lane), v);
     }
     if (sums) {
       for (int k = wid; k < 8; k += nwarp) {
