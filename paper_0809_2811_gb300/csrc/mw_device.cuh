@@ -24,6 +24,8 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "mw_quotient.h"
+
 namespace mw {
 
 constexpr double kKB = 0.0019872042586408316;  // kcal/mol/K
@@ -768,20 +770,6 @@ struct LdShared {
   __device__ static T get(const T& v) { return v; }
 };
 
-// a / b (FP64) from an FP32 reciprocal and two Newton steps: relative error
-// below 1e-13 in five FP64 operations.  The library division takes several
-// times that, and GB300 issues an FP64 instruction every ~25 cycles even for
-// one lane: with five divisions the isobaric tail took 5.5 us per step.  Its
-// callers round the quotient to FP32.  Divisors outside FP32's range divide.
-__device__ __forceinline__ double div_newton(double a, double b) {
-  const float bf = (float)b;
-  if (!(fabsf(bf) > 1e-30f && fabsf(bf) < 1e30f)) return a / b;
-  double r = (double)__frcp_rn(bf);
-  r = fma(r, fma(-b, r, 1.0), r);
-  r = fma(r, fma(-b, r, 1.0), r);
-  return a * r;
-}
-
 // Isotropic barostat (Sec. II.B, read as the Martyna-Tobias-Klein form):
 // half step on its momentum, pe += dt/2 [(1 + 3/N_df) 2 KE + tr(W) - 3 P V],
 // and the friction on the velocities, v *= exp(-dt/2 (1 + 3/N_df) pe/W),
@@ -791,7 +779,7 @@ __device__ __forceinline__ void baro_half(const Integ& I, const Box& bx, double 
   pe += 0.5 * I.dt * (bx.a3 * 2.0 * ke + trw - 3.0 * I.p_ext * Ld::get(bx.volume));
 }
 __device__ __forceinline__ float baro_friction(const Integ& I, const Box& bx, double pe) {
-  return expm1f((float)div_newton(-0.5 * I.dt * bx.a3 * pe, bx.W));
+  return expm1f((float)quotient(-0.5 * I.dt * bx.a3 * pe, bx.W));
 }
 
 // The box of the coming step: every edge scaled by e^u, u = dt pe/W, during
@@ -807,7 +795,7 @@ __device__ __forceinline__ float baro_friction(const Integ& I, const Box& bx, do
 // Returns bit 0: the margin asks for a rebuild, bit 1: the box left its grid.
 template <class Ld>
 __device__ int npt_geometry_of(const Integ& I, Box& bx, BoxState& st, double pe) {
-  const float u = (float)div_newton(I.dt * pe, bx.W);
+  const float u = (float)quotient(I.dt * pe, bx.W);
   const float eu = expm1f(u);
   const float fdr = fabsf(u) > 1e-3f ? -expm1f(-u) / u : fmaf(u, fmaf(u, 1.0f / 6.0f, -0.5f), 1.0f);
   const float dt64 = (float)(I.dt * 18446744073709551616.0);  // dt 2^64
@@ -820,7 +808,7 @@ __device__ int npt_geometry_of(const Integ& I, Box& bx, BoxState& st, double pe)
     const int nc = bx.nc[k];
     if (Ln < 2.0 * I.rlist || (nc >= 4 && Ln < nc * (double)I.rlist) || Ln >= (nc + 1) * kCellGrow * I.rlist) out = 2;
   }
-  const float c = (float)div_newton(bx.Ln[0], Ld::get(st.Lb));
+  const float c = (float)quotient(bx.Ln[0], Ld::get(st.Lb));
   const float m = I.skin - I.rlist * fmaxf(0.0f, 1.0f - c);
   if (m < 0.5f * I.skin) {
     st.rebuild = 1;
