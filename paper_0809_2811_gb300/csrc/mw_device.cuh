@@ -1794,7 +1794,8 @@ __device__ __forceinline__ int force_group(const Dev& d, const FParams& P, float
     } else {
       in = leg_terms(r2, P, lt);
     }
-    if (!in) {  // FP32 rounding put it on the cutoff (or past its pair's): contributes nothing
+    if (!in) {  // FP32 rounding put it on the cutoff (or past its pair's): contributes nothing (several
+                // species: the second record's r is 0 from phase A)
       (kSp ? *ue_p : *ax_p) = make_float4(0.f, 0.f, 0.f, 0.f);
       continue;
     }
@@ -1880,7 +1881,7 @@ __device__ __forceinline__ int force_group(const Dev& d, const FParams& P, float
     for (int l = g; l < nstage; l += KG) {
       const float4 uj = ue[at(l)];
       const float4 xj = aux[at(l)];
-      if (uj.w == 0.f) continue;  // leg dropped in phase B
+      if (xj.z == 0.f) continue;  // leg dropped in phase B
       const int wj = __float_as_int(xj.w);
       const float2* stj = stc + (wj >> 28) * nsp;
       const float r = xj.z;
@@ -1950,8 +1951,10 @@ __device__ __forceinline__ int force_group(const Dev& d, const FParams& P, float
     const float4 rec = ue[at(l)];
     const float4 xj = aux[at(l)];
     // the leg: its unit vector u, ee, -1/2 dphi, nde, 2 / r, its vector and partner
+    // (not ee: it is 0 where lambda is, or where exp(gamma sigma / (r - a sigma))
+    // underflows, and such a leg has its pair virial still)
     const float ee = kSp ? rec.w : xj.x;
-    if (ee == 0.f) continue;  // leg dropped in phase B
+    if ((kSp ? xj.z : xj.w) == 0.f) continue;  // leg dropped in phase B: r, or 1 / r, left 0
     const float hd = kSp ? xj.x : xj.y, nde = kSp ? xj.y : xj.z;
     const float tr = 2.0f * (kSp ? rcp_approx(xj.z) : xj.w);
     const float3 uj = kSp ? make_float3(rec.x, rec.y, rec.z) : make_float3(rec.x * xj.w, rec.y * xj.w, rec.z * xj.w);
