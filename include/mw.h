@@ -140,7 +140,8 @@ typedef struct mw_info {
   int force_lanes;           /* launch shape of the per-phase force kernel: lanes per centre atom ... */
   int force_blocks_per_sm;   /* ... and the co-resident blocks per SM its register budget allows */
   int force_owner;           /* 1: owner-computes (two passes, no per-leg scatter); 0: red.global scatter */
-  int pad_;
+  int cluster_blocks;        /* mw_step's last persistent run: blocks per box of the cluster form; 0: the grid-wide
+                                form, or another engine */
 } mw_info;
 
 typedef struct mw_system mw_system;
@@ -347,6 +348,14 @@ mw_status mw_energy_forces_vjp(mw_system* s, const float* dL_dF_dev, float* dL_d
  * (MW_EINVAL) while several species are set, and mw_set_species refuses
  * several species while it is selected. */
 mw_status mw_set_engine(mw_system* s, int engine);
+
+/* Diagnostics: the form that mw_step's persistent engine takes.  blocks = 0
+ * (the default): the library picks by size; 1, 2, 4, 8 or 16: clusters of that
+ * many blocks per box (512 atoms a block at most: MW_EINVAL if the largest box
+ * does not fit), wherever the cluster form can run at all (two steps or more,
+ * one species, no term counts or phase marks); -1: the grid-wide form.  Results
+ * agree to rounding; mw_info.cluster_blocks tells what ran. */
+mw_status mw_set_cluster_blocks(mw_system* s, int blocks);
 
 /* Sets the neighbour-list width (slots per atom, >= 1) and marks the list
  * stale; a width too small is grown again on the next build.  The library's

@@ -129,6 +129,8 @@ struct mw_system {
   // its cluster form: one buffer for the box order and the per-box progress
   int* clu_order = nullptr;
   bool clu_resume = false;  // the next launch goes on with boxes that stopped on their own steps
+  int clu_want = 0;         // mw_set_cluster_blocks: 0 by size, -1 never
+  int clu_used = 0;         // blocks per box of the last run (0: the grid-wide form, or another engine)
   bool clu_left = false;    // the last run ended with a box flagged for a build
   std::vector<int> cell_box_host;
   std::vector<void*> allocs;
@@ -1598,11 +1600,12 @@ mw_status mw_step(mw_system* s, const mw_integrator* integ, int nsteps, mw_therm
     if (eng == MW_ENGINE_PERSISTENT && !persistent_available(s)) eng = MW_ENGINE_GRAPH;
     s->engine_used = eng;
     CluConfig clu;
+    const bool clustered = eng == MW_ENGINE_PERSISTENT && cluster_config(s, nsteps, &clu);
+    s->clu_used = clustered ? clu.blocks : 0;
     s->clu_left = false;
-    st = eng == MW_ENGINE_PERSISTENT
-             ? (cluster_config(s, nsteps, &clu) ? run_cluster_engine(s, clu, nsteps, last, &fetched)
-                                        : run_persistent_engine(s, nsteps, last, &fetched))
-             : run_graph_engine(s, nsteps, last, &fetched, eng == MW_ENGINE_PLAIN);
+    st = clustered                     ? run_cluster_engine(s, clu, nsteps, last, &fetched)
+         : eng == MW_ENGINE_PERSISTENT ? run_persistent_engine(s, nsteps, last, &fetched)
+                                       : run_graph_engine(s, nsteps, last, &fetched, eng == MW_ENGINE_PLAIN);
     s->g_known_valid = false;
     if (st != MW_OK) {
       s->forces_valid = false;  // the state of an interrupted step is not a state to report forces of
@@ -1612,7 +1615,7 @@ mw_status mw_step(mw_system* s, const mw_integrator* integ, int nsteps, mw_therm
     s->list_built = true;
     // the steps built every row, but for boxes that had finished theirs
     // when the cluster form grew the rows: those are flagged still
-    s->rows_stale = s->rows_stale && eng == MW_ENGINE_PERSISTENT && s->clu_left;
+    s->rows_stale = s->rows_stale && s->clu_left;
   }
   if (last && !fetched) return mw_get_thermo(s, last);
   return MW_OK;
@@ -1630,6 +1633,7 @@ mw_status mw_step_async(mw_system* s, const mw_integrator* integ, int nsteps) {
   if (eng == MW_ENGINE_AUTO) eng = auto_engine(s);
   if (eng == MW_ENGINE_PERSISTENT && !persistent_available(s)) eng = MW_ENGINE_GRAPH;
   s->engine_used = eng;
+  s->clu_used = 0;  // (the cluster form belongs to mw_step)
   if ((st = prime_thermostat(s)) != MW_OK) return st;
   s->record_pending = true;
   if (eng == MW_ENGINE_PERSISTENT) return enqueue_persistent(s, nsteps, false);
@@ -1718,6 +1722,16 @@ mw_status mw_set_engine(mw_system* s, int engine) {
   return MW_OK;
 }
 
+mw_status mw_set_cluster_blocks(mw_system* s, int blocks) {
+  if (!s || blocks < -1 || blocks > kCluMax || (blocks & (blocks - 1) && blocks > 0))
+    return fail(MW_EINVAL, "cluster blocks must be -1, 0, 1, 2, 4, 8 or 16");
+  for (const Box& b : s->boxes)
+    if (blocks > 0 && b.n > blocks * kCluThreads)
+      return fail(MW_EINVAL, "a box of %d atoms does not fit %d blocks of %d", b.n, blocks, kCluThreads);
+  s->clu_want = blocks;
+  return MW_OK;
+}
+
 mw_status mw_set_nbr_width(mw_system* s, int width) {
   if (!s || width < 1) return fail(MW_EINVAL, "bad width");
   mw_status st;
@@ -1754,6 +1768,7 @@ mw_status mw_get_info(mw_system* s, mw_info* out) {
   out->force_lanes = force_shape_lanes(s->force_shape);
   out->force_blocks_per_sm = force_shape_blocks(s->force_shape);
   out->force_owner = force_shape_owner(s->force_shape) ? 1 : 0;
+  out->cluster_blocks = s->clu_used;
   return MW_OK;
 }
 

@@ -28,7 +28,7 @@ EXPORTS = (
     "mw_params_default", "mw_system_create", "mw_batch_create", "mw_system_destroy", "mw_set_state",
     "mw_set_state_dev", "mw_get_state", "mw_get_state_dev", "mw_set_params", "mw_build_neighbors",
     "mw_get_neighbors", "mw_energy_forces", "mw_energy_forces_dev", "mw_step", "mw_get_thermo",
-    "mw_energy_forces_vjp", "mw_set_engine", "mw_set_nbr_width", "mw_autotune", "mw_get_info",
+    "mw_energy_forces_vjp", "mw_set_engine", "mw_set_cluster_blocks", "mw_set_nbr_width", "mw_autotune", "mw_get_info",
     "mw_set_count_terms", "mw_forces_async", "mw_step_async", "mw_sync", "mw_energy_forces_noalloc", "mw_set_skin", "mw_set_force_shape", "mw_phase_times",
     "mw_pair_histogram", "mw_angle_histogram", "mw_get_unwrapped", "mw_get_box", "mw_set_species",
     "mw_checkpoint_size", "mw_checkpoint_save", "mw_checkpoint_load", "mw_set_wait_limit",
@@ -70,7 +70,7 @@ class mw_info(ctypes.Structure):
                 ("r_list", ctypes.c_double), ("npairs", ctypes.c_int64), ("ntriplets", ctypes.c_int64),
                 ("rebuild_steps", ctypes.c_int64), ("regrids", ctypes.c_int64), ("species", ctypes.c_int),
                 ("species_moments", ctypes.c_int), ("force_lanes", ctypes.c_int), ("force_blocks_per_sm", ctypes.c_int),
-                ("force_owner", ctypes.c_int), ("pad_", ctypes.c_int)]
+                ("force_owner", ctypes.c_int), ("cluster_blocks", ctypes.c_int)]
 
 
 class MWError(RuntimeError):
@@ -112,6 +112,7 @@ def lib():
             "mw_get_thermo": [P, ctypes.POINTER(mw_thermo)],
             "mw_energy_forces_vjp": [P, P, P, dp],
             "mw_set_engine": [P, ctypes.c_int],
+            "mw_set_cluster_blocks": [P, ctypes.c_int],
             "mw_set_nbr_width": [P, ctypes.c_int],
             "mw_autotune": [P, ctypes.POINTER(mw_integrator), ctypes.c_int, ip],
             "mw_get_info": [P, ctypes.POINTER(mw_info)],
@@ -343,6 +344,11 @@ def mw_energy_forces_vjp(h: int, dL_dF_dev, dL_dx_dev, nbox: int = 1):
 
 def mw_set_engine(h: int, engine: int):
     _check(lib().mw_set_engine(h, engine))
+
+
+def mw_set_cluster_blocks(h: int, blocks: int):
+    """Form of mw_step's persistent engine: 0 by size, 1-16 blocks per box, -1 grid-wide."""
+    _check(lib().mw_set_cluster_blocks(h, int(blocks)))
 
 
 def mw_set_nbr_width(h: int, width: int):

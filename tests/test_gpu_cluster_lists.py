@@ -59,6 +59,7 @@ def _overflowed(mwlib):
     th = s.step(STEPS, **KW)
     assert all(t["step"] == STEPS for t in th)
     assert s.info()["nbr_width"] > fit  # the rows were grown during the run
+    assert s.info()["cluster_blocks"] > 0
     return s, boxes
 
 

@@ -29,7 +29,7 @@ def test_kinetic_energy_is_exact_beyond_a_warp(mwlib):
         s.set_engine(2)
         s.set_state(np.tile(x0, (nbox, 1)), v.reshape(-1, 3))
         th = s.step(2, dt=1.0)
-        assert s.info()["engine"] == 2
+        assert s.info()["cluster_blocks"] in (1, 2)  # blocks of 350 atoms or more
     finally:
         s.close()
     want = (a.astype(np.int64) ** 2).sum(axis=1) * 2.0 ** -21

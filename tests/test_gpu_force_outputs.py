@@ -54,6 +54,7 @@ def test_forces_of_the_step_that_left_the_grid(mwlib, orc, engine):
         s.energy_forces()  # (other forces, energies and virials in the staging buffers)
         s.step(k, **KW)
         assert s.info()["regrids"] == 0
+        assert (s.info()["cluster_blocks"] > 0) == (engine == "cluster")
         x, _ = s.get_state()
         box = s.box()[0]
         f, e, w = s.energy_forces()

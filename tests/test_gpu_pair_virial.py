@@ -60,6 +60,7 @@ def test_pair_virial_of_the_persistent_engine(mwlib, orc, which, grid_wide):
         s.set_state(np.tile(x, (4, 1)), np.tile(v, (4, 1)))
         th = s.step(2, dt=10.0)
         xg, _ = s.get_state()
+        assert (s.info()["cluster_blocks"] == 0) == grid_wide
     finally:
         s.close()
     for b in range(4):
