@@ -271,10 +271,12 @@ __device__ __forceinline__ double fraction_times(unsigned long long f, double L)
   return __longlong_as_double(__double_as_longlong(__ull2double_rn(h)) + (scale << 52));
 }
 
-// FP32 to FP64, exact (zero for a subnormal).
+// FP32 to FP64, exact (a subnormal, which hardly any call meets, by the
+// conversion instruction).
 __device__ __forceinline__ double widen(float f) {
   const uint32_t u = __float_as_uint(f);
   const uint32_t ex = (u >> 23) & 0xffu;
+  if (ex == 0u && (u & 0x7fffffu)) return (double)f;
   const uint32_t hi = ex == 0u ? 0u : ((ex == 255u ? 2047u : ex + 896u) << 20) | ((u & 0x7fffffu) >> 3);
   return __hiloint2double((int)((u & 0x80000000u) | hi), ex == 0u ? 0 : (int)(u << 29));
 }
