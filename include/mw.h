@@ -378,8 +378,10 @@ mw_status mw_set_skin(mw_system* s, double skin);
  * current one) and persistent grid size - each from the same saved state
  * (positions, velocities and thermostat state are restored exactly between
  * candidates and at the end), keeps the fastest by GPU time as the AUTO
- * engine and the skin, and writes it to *best_engine (may be NULL).  The
- * choice is cached per device name and system signature in the text file
+ * engine and the skin, and writes it to *best_engine (may be NULL).  Where
+ * mw_step's persistent engine takes its cluster form, that form is timed for
+ * mw_step, and mw_step_async (which has no cluster form) gets its own choice
+ * of engine and grid size at the same skin.  The choice is cached per device name and system signature in the text file
  * named by the environment variable MW_AUTOTUNE_CACHE, when set.  The
  * persistent engine's force phase keeps its own shape (4 lanes per centre,
  * the register budget of the cooperative kernel). */

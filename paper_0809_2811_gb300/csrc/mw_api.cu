@@ -114,7 +114,7 @@ struct mw_system {
   size_t ana_cap = 0;
   long long host_step = 0;
   int engine = MW_ENGINE_AUTO, engine_used = MW_ENGINE_GRAPH;
-  int tuned_engine = -1;
+  int tuned_engine = -1, tuned_async = -1;  // the autotuner's engines for mw_step and mw_step_async
   int force_shape = 0;  // launch shape of k_force (force_shape_lanes / force_shape_blocks)
   int count_terms = 0;
   long long npairs = 0, ntrip = 0;
@@ -1579,8 +1579,8 @@ mw_status mw_forces_async(mw_system* s) {
 // 1925, 230000 2632 / 2737; 38 boxes of 4000 2325 / 2262, 50 2728 / 2653; 256
 // uneven boxes of 1.16 10^6 atoms 11808 / 10455.  Isobaric runs stay: the
 // persistent tail is quicker (64000 atoms 1826 / 2696).
-static int auto_engine(const mw_system* s) {
-  if (s->tuned_engine >= 0) return s->tuned_engine;
+static int auto_engine(const mw_system* s, bool async) {
+  if (s->tuned_engine >= 0) return async ? s->tuned_async : s->tuned_engine;
   const int most = s->nbox <= kOwnBoxes ? 200000 : 150000;
   return s->N > most && s->integ.kind != TH_NPT ? MW_ENGINE_GRAPH : MW_ENGINE_PERSISTENT;
 }
@@ -1596,7 +1596,7 @@ mw_status mw_step(mw_system* s, const mw_integrator* integ, int nsteps, mw_therm
   bool fetched = false;  // the run's last record came back with its final status read
   if (nsteps > 0) {
     int eng = s->engine;
-    if (eng == MW_ENGINE_AUTO) eng = auto_engine(s);
+    if (eng == MW_ENGINE_AUTO) eng = auto_engine(s, false);
     if (eng == MW_ENGINE_PERSISTENT && !persistent_available(s)) eng = MW_ENGINE_GRAPH;
     s->engine_used = eng;
     CluConfig clu;
@@ -1630,7 +1630,7 @@ mw_status mw_step_async(mw_system* s, const mw_integrator* integ, int nsteps) {
   if ((st = ensure_forces(s)) != MW_OK) return st;
   if (nsteps == 0) return MW_OK;
   int eng = s->engine;
-  if (eng == MW_ENGINE_AUTO) eng = auto_engine(s);
+  if (eng == MW_ENGINE_AUTO) eng = auto_engine(s, true);
   if (eng == MW_ENGINE_PERSISTENT && !persistent_available(s)) eng = MW_ENGINE_GRAPH;
   s->engine_used = eng;
   s->clu_used = 0;  // (the cluster form belongs to mw_step)
