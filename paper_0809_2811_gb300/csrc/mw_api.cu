@@ -1570,19 +1570,29 @@ mw_status mw_forces_async(mw_system* s) {
 }
 
 // The engine of MW_ENGINE_AUTO where no autotuner has chosen: the persistent
-// one, and the graph engine above 200000 atoms (150000 in batches whose
-// thermostats the last block evaluates).  The grid-wide kernel runs every
-// phase at the force phase's 20 warps an SM; for large systems the separate
-// kernels' 32 are worth more than the launches between them.  20 steps, skin
-// 1 A, us, persistent / graph: 65536 atoms 932 / 1172, 150000 1888 / 1934,
-// 200000 2232 / 2280, 230000 2743 / 2730; without a thermostat 150000 1796 /
-// 1925, 230000 2632 / 2737; 38 boxes of 4000 2325 / 2262, 50 2728 / 2653; 256
-// uneven boxes of 1.16 10^6 atoms 11808 / 10455.  Isobaric runs stay: the
-// persistent tail is quicker (64000 atoms 1826 / 2696).
+// one up to a number of atoms, the graph engine above it.  The grid-wide kernel
+// runs every phase at the force phase's 20 warps an SM; for large systems the
+// separate kernels' 32 are worth more than the launches between them.  The line
+// falls with the number of boxes (some box builds its list in more of the
+// steps, and a build is where the separate kernels gain most) and lies higher
+// without a thermostat, where a persistent step has one barrier less.  Graph
+// over grid-wide persistent time, 20 steps, skin 1 A, by boxes and 1000 atoms
+// in all:
+//   Nose-Hoover   1: 210 1.03, 262 1.02, 310 0.98, 350 0.98, 500 0.93; 7: 280 1.03;
+//                 9: 160 1.06, 240 1.02, 300 1.01; 16: 160 1.03, 240 1.02, 300 0.98;
+//                 24: 160 1.01, 200 0.98, 300 0.98; 40: 160 1.00, 240 0.98;
+//                 80 to 400: 100 0.99 to 1.05, 160 0.96 to 0.99, 400 0.91 to 0.94
+//   NVE           1: 210 1.08, 350 1.02, 375 1.00, 430 0.98; 9: 160 1.12, 300 1.05;
+//                 16: 300 1.02; 40: 240 1.02, 300 1.00; 130 to 520: 160 1.02 to 1.04,
+//                 260 0.99 to 1.01, 400 0.97
+// Isobaric runs stay: the persistent tail is quicker (64000 atoms 1826 us
+// against 2696).
 static int auto_engine(const mw_system* s, bool async) {
   if (s->tuned_engine >= 0) return async ? s->tuned_async : s->tuned_engine;
-  const int most = s->nbox <= kOwnBoxes ? 200000 : 150000;
-  return s->N > most && s->integ.kind != TH_NPT ? MW_ENGINE_GRAPH : MW_ENGINE_PERSISTENT;
+  if (s->integ.kind == TH_NPT) return MW_ENGINE_PERSISTENT;
+  const int most = s->integ.kind == TH_NVE ? std::max(220000, 400000 - 2500 * std::min(s->nbox, 100))
+                                           : std::max(130000, 310000 - 3500 * std::min(s->nbox, 100));
+  return s->N > most ? MW_ENGINE_GRAPH : MW_ENGINE_PERSISTENT;
 }
 
 mw_status mw_step(mw_system* s, const mw_integrator* integ, int nsteps, mw_thermo* last) {
