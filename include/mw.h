@@ -374,8 +374,8 @@ mw_status mw_set_skin(mw_system* s, double skin);
  * blocks per SM with red.global scatter, and 4 x 8 owner-computes; see
  * mw_set_force_shape) is timed over 10 force calls on the current state and
  * the fastest kept.  Then it runs `steps` steps for each candidate configuration
- * - engine (graph / persistent), skin (0.7x, 1x, 1.4x, 1.8x, 2.2x, 2.6x the
- * current one) and persistent grid size - each from the same saved state
+ * - engine (graph / persistent), skin (0.7x, 1x, 1.2x, 1.4x, 1.6x, 1.8x, 2x,
+ * 2.2x, 2.6x the current one) and persistent grid size - each from the same saved state
  * (positions, velocities and thermostat state are restored exactly between
  * candidates and at the end), keeps the fastest by GPU time as the AUTO
  * engine and the skin, and writes it to *best_engine (may be NULL).  Where

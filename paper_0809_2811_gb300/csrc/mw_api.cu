@@ -2,8 +2,9 @@
 //
 // Host side: validates arguments, owns device buffers, sequences the kernels
 // of mw_device.cuh on the system's stream, captures one MD step into a CUDA
-// graph (graph engine) or launches the persistent cooperative kernel
-// (persistent engine), and recovers from neighbour-list overflow.
+// graph (graph engine) or launches a kernel that runs many steps (persistent
+// engine: one cooperative kernel over the whole grid, or one thread-block
+// cluster per box), and recovers from neighbour-list overflow.
 #include <cuda_runtime.h>
 
 #include <algorithm>

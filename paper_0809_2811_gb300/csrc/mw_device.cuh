@@ -224,7 +224,8 @@ __device__ __forceinline__ unsigned long long frac64_of(double s) {
 // result is the same (61 and 36 us).
 
 // Box fraction of the coordinate x in an edge L, rl = 1 / L: round(x / L 2^64)
-// mod 2^64 (the quotient to its last FP64 bit), and the whole edges below it.
+// mod 2^64 (the quotient corrected by its own remainder, Markstein's form: to
+// its last FP64 bit), and the whole edges below it.
 __device__ __forceinline__ unsigned long long box_fraction(double x, double L, double rl, int& image) {
   double q = x * rl;
   q = fma(fma(-q, L, x), rl, q);
