@@ -1564,7 +1564,7 @@ mw_status mw_forces_async(mw_system* s) {
   if (!s) return fail(MW_EINVAL, "system is NULL");
   mw_status st;
   if ((st = ensure_rows(s)) != MW_OK) return st;
-  k_prep_force<<<div_up(std::max(s->N, s->nbox), kThreads), kThreads, 0, s->stream>>>(s->d, 1);
+  k_prep_force<<<div_up(std::max(s->N, s->nbox), kThreads), kThreads, 0, s->stream>>>(s->d, 3);
   launch_force(s);
   MW_CUDA(cudaGetLastError());
   return MW_OK;

@@ -2635,9 +2635,13 @@ __host__ __device__ inline int kick_blocks(int n, int threads, int items = 1) {
   return (n + per - 1) / per;
 }
 
-// The same with the forces (mode 1, 2), a pending half-kick applied with the
+// The same with the forces (mode 1 to 3), a pending half-kick applied with the
 // old ones first (mode 2: the host clears Global::pend after the launch).
+// Mode 3 leaves everything as it is under a status, under which no force
+// kernel runs either: the valid forces of an isobaric box that left its cell
+// grid stay those of its last step.
 __global__ void k_prep_force(Dev d, int mode) {
+  if (mode == 3 && *(volatile int*)&d.g->status) return;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   prep_box(d, i);
   if (mode > 0 && i < d.N) {

@@ -71,6 +71,35 @@ def test_forces_of_the_step_that_left_the_grid(mwlib, orc, engine):
     compare(f"after the grid was left [{engine}, device]", fd.cpu().numpy(), ed.cpu().numpy()[0], wd.cpu().numpy()[0], ref)
 
 
+def test_asynchronous_force_call_after_the_grid_was_left(mwlib, orc):
+    """mw_forces_async changes nothing until mw_sync has laid the grid out
+    again; the forces, and the steps that take them, are those of the run."""
+    k = _leaving_step(mwlib)
+    x0, v0, box0 = _collapsing()
+    s = _system(mwlib, "cluster")
+    try:
+        s.step(k, **KW)
+        x, _ = s.get_state()
+        box = s.box()[0]
+        mwlib.mw_forces_async(s.h)
+        with pytest.raises(mwlib.MWError) as ei:
+            mwlib.mw_sync(s.h)
+        assert ei.value.status == mwlib.MW_EGRID
+        f, e, w = s.energy_forces()
+        mwlib.mw_forces_async(s.h)
+        mwlib.mw_sync(s.h)
+        f2, _, _ = s.energy_forces()
+        th = s.step(2, **KW)[0]
+    finally:
+        s.close()
+    ref = orc.energy_forces(x, box)
+    compare("asynchronous call, grid left", f, e[0], w[0], ref)
+    compare("asynchronous call, grid laid out", f2, e[0], w[0], ref, force_only=True)
+    _, _, bo, _, tho = orc.md_npt(x0, v0, box0, k + 2, dt=10.0, T0=250.0, tau=200.0, p_atm=0.0, tau_p=500.0)
+    assert th["pe"] == pytest.approx(tho[-1, 0], rel=1e-6)  # as in test_gpu_npt.py
+    assert th["ke"] == pytest.approx(tho[-1, 3], rel=3e-6)
+
+
 @pytest.mark.parametrize("synced", [False, True])
 def test_force_call_after_a_failed_asynchronous_run_reports_it(mwlib, synced):
     torch = pytest.importorskip("torch")
