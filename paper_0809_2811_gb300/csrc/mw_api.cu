@@ -1586,13 +1586,15 @@ mw_status mw_forces_async(mw_system* s) {
 //   NVE           1: 210 1.08, 350 1.02, 375 1.00, 430 0.98; 9: 160 1.12, 300 1.05;
 //                 16: 300 1.02; 40: 240 1.02, 300 1.00; 130 to 520: 160 1.02 to 1.04,
 //                 260 0.99 to 1.01, 400 0.97
-// Isobaric runs stay: the persistent tail is quicker (64000 atoms 1826 us
+// and no lower, since mw_step runs batches of small boxes in clusters: 100
+// boxes of 1000 atoms 1974 us with the graph engine, 1927 grid-wide, 1642 in
+// clusters.  Isobaric runs stay: the persistent tail is quicker (64000 atoms 1826 us
 // against 2696).
 static int auto_engine(const mw_system* s, bool async) {
   if (s->tuned_engine >= 0) return async ? s->tuned_async : s->tuned_engine;
   if (s->integ.kind == TH_NPT) return MW_ENGINE_PERSISTENT;
   const int most = s->integ.kind == TH_NVE ? std::max(220000, 400000 - 2500 * std::min(s->nbox, 100))
-                                           : std::max(130000, 310000 - 3500 * std::min(s->nbox, 100));
+                                           : std::max(150000, 310000 - 3500 * std::min(s->nbox, 100));
   return s->N > most ? MW_ENGINE_GRAPH : MW_ENGINE_PERSISTENT;
 }
 

@@ -12,6 +12,7 @@ NVE, NH, NPT = 0, 2, 3
 CASES = [  # boxes, atoms a box, thermostat, engine (1 graph, 2 persistent)
     (1, 262144, NVE, 2), (1, 262144, NH, 2), (1, 262144, NPT, 2), (1, 350000, NH, 1), (1, 430000, NVE, 1),
     (9, 17777, NVE, 2), (9, 17777, NH, 2), (40, 7500, NH, 1), (130, 2000, NH, 1), (320, 500, NVE, 2),
+    (145, 1000, NH, 2),
 ]
 
 
