@@ -22,5 +22,7 @@ def test_form_by_size(mwlib, nbox, n, thermostat, clustered):
         s.set_state(np.tile(x, (nbox, 1)))
         s.step(2, dt=5.0, thermostat=thermostat, T0=200.0)
         assert (s.info()["cluster_blocks"] > 0) == clustered
+        if (nbox, n) == (200, 500):
+            assert s.info()["cluster_blocks"] == 2
     finally:
         s.close()
